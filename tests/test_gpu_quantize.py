@@ -43,6 +43,15 @@ def test_codes_and_scales_match_the_oracle_bit_for_bit(marlin, K, N, G, n_grid, 
     assert np.array_equal(to_host(q).view(np.uint32), inputs.kpack(Q_ref))
 
 
+# groups above 128 rows: one candidate per warp (few blocks) or a pair of them (many), more candidates than one round of
+# warps takes, odd counts, tiles of 64 rows that wrap the ring
+@pytest.mark.parametrize("K,N,G,n_grid,n_cand", [
+    (512, 64, 256, 40, 37), (1024, 2048, 256, 40, 35), (1024, 4096, 256, 20, 10), (1024, 2112, -1, 20, 10),
+    (256, 64, -1, 20, 2), (3072, 192, 1536, 20, 17)])
+def test_long_groups_match_the_oracle_bit_for_bit(marlin, K, N, G, n_grid, n_cand):
+    test_codes_and_scales_match_the_oracle_bit_for_bit(marlin, K, N, G, n_grid, n_cand)
+
+
 def test_plain_rounding_versus_search_on_outlier_groups(marlin):
     import torch
     W = _weights(1024, 256, 9, outliers=False)
