@@ -34,15 +34,6 @@
 namespace marlin_b200 {
 namespace {
 
-// word `wi` (0..1023) of chunk (kb, nb), nibble p -> matrix position
-__device__ __forceinline__ void decode_position(int wi, int p, int kb, int nb, int* k, int* n) {
-  int w = wi & 3, lane = (wi >> 2) & 31, i = wi >> 7;
-  int g = lane >> 2, c = ((lane & 3) - (g >> 1)) & 3, j = i >> 1, b = i & 1;  // slot = (c + g/2) % 4
-  int o = 2 * (p & 3) + (p >> 2);
-  *n = 64 * nb + 16 * j + 8 * b + g;
-  *k = 128 * kb + 64 * (w >> 1) + 16 * c + 8 * (w & 1) + o;
-}
-
 // chunk index <-> (kb, nb)
 __device__ __forceinline__ long long chunk_index(int kb, int nb, int KB, int nb64) {
   int sc = nb >> 2;
@@ -64,68 +55,39 @@ __device__ __forceinline__ void chunk_coords(long long chunk, int KB, int nb64, 
   }
 }
 
-__global__ void pack_weights_kernel(const uint32_t* __restrict__ q, uint32_t* __restrict__ wq, int K, int N) {
-  long long total = (long long)K * N / 8;
-  for (long long wi = blockIdx.x * (long long)blockDim.x + threadIdx.x; wi < total;
-       wi += (long long)gridDim.x * blockDim.x) {
-    int nb64 = N / 64;
-    int kb, nb;
-    chunk_coords(wi >> 10, K / 128, nb64, &kb, &nb);
-    uint32_t out = 0;
-#pragma unroll
-    for (int p = 0; p < 8; ++p) {
-      int k, n;
-      decode_position((int)(wi & 1023), p, kb, nb, &k, &n);
-      uint32_t code = (q[(size_t)(k >> 3) * N + n] >> (4 * (k & 7))) & 15u;
-      out |= code << (4 * p);
-    }
-    wq[wi] = out;
-  }
+// The nibbles of a canonical word (row offset o in nibble o) in the packed order (nibble (o >> 1) + 4 * (o & 1)), and back.
+__device__ __forceinline__ uint32_t even_nibbles(uint32_t w) {  // nibbles 0, 2, 4, 6 side by side in the low half
+  w &= 0x0f0f0f0fu;
+  w = (w | (w >> 4)) & 0x00ff00ffu;
+  return (w | (w >> 8)) & 0xffffu;
+}
+__device__ __forceinline__ uint32_t spread_nibbles(uint32_t h) {  // its inverse
+  h = (h | (h << 8)) & 0x00ff00ffu;
+  return (h | (h << 4)) & 0x0f0f0f0fu;
+}
+__device__ __forceinline__ uint32_t to_packed_word(uint32_t w) { return even_nibbles(w) | (even_nibbles(w >> 4) << 16); }
+__device__ __forceinline__ uint32_t to_canonical_word(uint32_t w) {
+  return spread_nibbles(w & 0xffffu) | (spread_nibbles(w >> 16) << 4);
 }
 
-__global__ void unpack_weights_kernel(const uint32_t* __restrict__ wq, uint32_t* __restrict__ q, int K, int N) {
-  long long total = (long long)K * N / 8;
-  int nb64 = N / 64;
-  for (long long qi = blockIdx.x * (long long)blockDim.x + threadIdx.x; qi < total;
-       qi += (long long)gridDim.x * blockDim.x) {
-    int n = (int)(qi % N);
-    int k8 = (int)(qi / N);
-    int nb = n >> 6, j = (n >> 4) & 3, b = (n >> 3) & 1, g = n & 7;
-    uint32_t out = 0;
-#pragma unroll
-    for (int jn = 0; jn < 8; ++jn) {
-      int k = 8 * k8 + jn;
-      int kb = k >> 7, h = (k >> 6) & 1, c = (k >> 4) & 3, u = (k >> 3) & 1, o = k & 7;
-      int p = (o >> 1) + 4 * (o & 1);
-      int lane = 4 * g + ((c + (g >> 1)) & 3), i = 2 * j + b, w = 2 * h + u;
-      long long wi = ((chunk_index(kb, nb, K / 128, nb64) * 8 + i) * 32 + lane) * 4 + w;
-      uint32_t code = (wq[wi] >> (4 * p)) & 15u;
-      out |= code << (4 * jn);
-    }
-    q[qi] = out;
-  }
+// scale at packed position x -> its canonical position
+__device__ __forceinline__ long long canonical_scale(long long x, int N, int sub) {
+  const int pos = (int)(x & 63);  // packed position inside the run of 64
+  const int g = pos >> 3, j = (pos >> 1) & 3, b = pos & 1;
+  const int c64 = 16 * j + 8 * b + g;  // column inside the run
+  if (sub == 1) return (x & ~63LL) + c64;
+  // packed [kb][tile][r][256]  <->  canonical row kb * sub + r, column 256 * tile + ...
+  const long long rec = x >> 8;  // (kb * NT + tile) * sub + r
+  const int r = (int)(rec % sub);
+  const long long kt = rec / sub;
+  const int NT = N / 256;
+  const long long kb = kt / NT, tile = kt % NT;
+  return (kb * sub + r) * (long long)N + tile * 256 + (x & 192) + c64;
 }
-
-__global__ void permute_scales_kernel(const uint16_t* __restrict__ in, uint16_t* __restrict__ out, long long total,
-                                      int N, int sub, bool inverse) {
-  for (long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x; x < total;
-       x += (long long)gridDim.x * blockDim.x) {
-    // x = packed position
-    const int pos = (int)(x & 63);  // packed position inside the run of 64
-    const int g = pos >> 3, j = (pos >> 1) & 3, b = pos & 1;
-    const int c64 = 16 * j + 8 * b + g;  // column inside the run
-    long long canon;
-    if (sub == 1) {
-      canon = (x & ~63LL) + c64;
-    } else {
-      // packed [kb][tile][r][256]  <->  canonical row kb * sub + r, column 256 * tile + ...
-      const long long rec = x >> 8;  // (kb * NT + tile) * sub + r
-      const int r = (int)(rec % sub);
-      const long long kt = rec / sub;
-      const int NT = N / 256;
-      const long long kb = kt / NT, tile = kt % NT;
-      canon = (kb * sub + r) * (long long)N + tile * 256 + (x & 192) + c64;
-    }
+__device__ __forceinline__ void permute_scales(const uint16_t* __restrict__ in, uint16_t* __restrict__ out, long long total,
+                                               int N, int sub, bool inverse, int block, int blocks) {
+  for (long long x = block * (long long)blockDim.x + threadIdx.x; x < total; x += (long long)blocks * blockDim.x) {
+    const long long canon = canonical_scale(x, N, sub);
     if (inverse)
       out[canon] = in[x];
     else
@@ -133,25 +95,65 @@ __global__ void permute_scales_kernel(const uint16_t* __restrict__ in, uint16_t*
   }
 }
 
+// Codes and scales of a dense layer in one launch: the first `code_blocks` blocks take the chunks, the others the scales.
+// A chunk is 16 canonical word rows x 64 columns, and every packed word is one canonical word with its nibbles permuted:
+// the block moves the chunk through shared memory so that both sides are read and written 16 bytes a thread in whole
+// lines.  Bound: DRAM, both buffers once.  (One thread per packed word that gathered its canonical word took 25 us on
+// 4096 x 11008, the scales another launch of 4 us; both together take 13 us now.)
+constexpr int kPackThreads = 256;
+__global__ void __launch_bounds__(kPackThreads)
+repack_dense_kernel(const uint4* __restrict__ src, uint4* __restrict__ dst, const uint16_t* __restrict__ s_src,
+                    uint16_t* __restrict__ s_dst, int K, int N, long long scales, int sub, int code_blocks, bool inverse) {
+  if ((int)blockIdx.x >= code_blocks) {
+    permute_scales(s_src, s_dst, scales, N, sub, inverse, blockIdx.x - code_blocks, gridDim.x - code_blocks);
+    return;
+  }
+  // rows padded by four words: the 32 words a warp takes by vectors (four rows, eight columns) lie in different banks
+  __shared__ __align__(16) uint32_t tile[16][kChunkN + 4];
+  const int t = threadIdx.x;
+  const int KB = K / kTileK, nb64 = N / kChunkN;
+  const int row = t >> 4, c4 = t & 15;  // by rows: four columns of a word row
+  // by vectors: vector t of the chunk holds rows 16c .. and 64 + 16c .. of column 8i + g, slot = (c + g / 2) % 4
+  const int i = t >> 5, g = (t & 31) >> 2, c = ((t & 3) - (g >> 1)) & 3;
+  const int col = 8 * i + g;
+  for (long long chunk = blockIdx.x; chunk < (long long)KB * nb64; chunk += code_blocks) {
+    int kb, nb;
+    chunk_coords(chunk, KB, nb64, &kb, &nb);
+    const size_t canon = (((size_t)kb * 16 + row) * N + (size_t)nb * kChunkN) / 4 + c4;
+    const size_t packed = (size_t)chunk * kPackThreads + t;
+    if (!inverse) {
+      *reinterpret_cast<uint4*>(&tile[row][4 * c4]) = src[canon];
+      __syncthreads();
+      uint4 v;
+      v.x = to_packed_word(tile[2 * c][col]);
+      v.y = to_packed_word(tile[2 * c + 1][col]);
+      v.z = to_packed_word(tile[8 + 2 * c][col]);
+      v.w = to_packed_word(tile[8 + 2 * c + 1][col]);
+      dst[packed] = v;
+    } else {
+      const uint4 v = src[packed];
+      tile[2 * c][col] = to_canonical_word(v.x);
+      tile[2 * c + 1][col] = to_canonical_word(v.y);
+      tile[8 + 2 * c][col] = to_canonical_word(v.z);
+      tile[8 + 2 * c + 1][col] = to_canonical_word(v.w);
+      __syncthreads();
+      dst[canon] = *reinterpret_cast<const uint4*>(&tile[row][4 * c4]);
+    }
+    __syncthreads();
+  }
+}
+
+__global__ void permute_scales_kernel(const uint16_t* __restrict__ in, uint16_t* __restrict__ out, long long total,
+                                      int N, int sub, bool inverse) {
+  permute_scales(in, out, total, N, sub, inverse, blockIdx.x, gridDim.x);
+}
+
 // zero points: the same permutation, uint8 codes on the canonical side and fp16 values on the packed side
 __global__ void permute_zeros_kernel(uint8_t* __restrict__ z, uint16_t* __restrict__ zq, long long total, int N, int sub,
                                      bool inverse) {
   for (long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x; x < total;
        x += (long long)gridDim.x * blockDim.x) {
-    const int pos = (int)(x & 63);
-    const int g = pos >> 3, j = (pos >> 1) & 3, b = pos & 1;
-    const int c64 = 16 * j + 8 * b + g;
-    long long canon;
-    if (sub == 1) {
-      canon = (x & ~63LL) + c64;
-    } else {
-      const long long rec = x >> 8;
-      const int r = (int)(rec % sub);
-      const long long kt = rec / sub;
-      const int NT = N / 256;
-      const long long kb = kt / NT, tile = kt % NT;
-      canon = (kb * sub + r) * (long long)N + tile * 256 + (x & 192) + c64;
-    }
+    const long long canon = canonical_scale(x, N, sub);
     if (inverse)
       z[canon] = (uint8_t)__half2float(__ushort_as_half(zq[x]));
     else
@@ -230,17 +232,15 @@ cudaError_t launch_permute_zeros(uint8_t* z, uint16_t* zq, int K, int N, int G, 
 
 cudaError_t launch_pack_dense(uint32_t* q, uint16_t* s, uint32_t* wq, uint16_t* sq, int K, int N, int G, bool inverse,
                               cudaStream_t stream) {
-  long long words = (long long)K * N / 8;
-  int threads = 256;
-  int blocks = (int)((words + threads - 1) / threads);
-  if (blocks > 148 * 16) blocks = 148 * 16;
-  if (!inverse)
-    pack_weights_kernel<<<blocks, threads, 0, stream>>>(q, wq, K, N);
-  else
-    unpack_weights_kernel<<<blocks, threads, 0, stream>>>(wq, q, K, N);
-  cudaError_t err = cudaGetLastError();
-  if (err != cudaSuccess) return err;
-  return launch_permute_scales(s, sq, K, N, G, inverse, stream);
+  const long long chunks = (long long)(K / kTileK) * (N / kChunkN), ns = (long long)(K / G) * N;
+  const int code_blocks = (int)(chunks < 148 * 16 ? chunks : 148 * 16);
+  const long long sb = (ns + kPackThreads - 1) / kPackThreads;
+  const int scale_blocks = (int)(sb < 148 * 2 ? sb : 148 * 2);
+  const int sub = G < kTileK ? kTileK / G : 1;
+  repack_dense_kernel<<<code_blocks + scale_blocks, kPackThreads, 0, stream>>>(
+      reinterpret_cast<const uint4*>(inverse ? wq : q), reinterpret_cast<uint4*>(inverse ? q : wq), inverse ? sq : s,
+      inverse ? s : sq, K, N, ns, sub, code_blocks, inverse);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_permute_scales(uint16_t* s, uint16_t* sq, int K, int N, int G, bool inverse, cudaStream_t stream) {
