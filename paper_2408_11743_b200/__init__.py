@@ -17,6 +17,7 @@ from .binding import (  # noqa: F401
     lib,
     mlp_swiglu,
     library_path,
+    native,
     new_workspace,
     pack,
     pack_sparse24,

@@ -1,4 +1,5 @@
-"""Builds libmarlin_b200.so (sm_100a only) next to this file with nvcc.
+"""Builds libmarlin_b200.so (sm_100a only) with nvcc and the extension module of the Python binding with g++, next to
+this file.
 
     python -m paper_2408_11743_b200.build [--force] [--verbose]
 
@@ -29,6 +30,30 @@ def _nvcc() -> str:
         if cand and (os.path.isabs(cand) and os.path.exists(cand) or not os.path.isabs(cand)):
             return cand
     return "nvcc"
+
+
+# the per-call part of the Python binding: host code against torch's C++ API
+NATIVE = os.path.join(_HERE, "_torch_binding.so")
+NATIVE_SOURCE = os.path.join(CSRC, "torch_binding.cpp")
+
+
+def build_native(force: bool = False, verbose: bool = False) -> str:
+    import sysconfig
+    deps = [NATIVE_SOURCE, os.path.abspath(__file__)]
+    if not force and os.path.exists(NATIVE) and all(os.path.getmtime(d) <= os.path.getmtime(NATIVE) for d in deps):
+        return NATIVE
+    import torch
+    t = os.path.dirname(torch.__file__)
+    cuda = os.path.dirname(os.path.dirname(_nvcc())) if os.path.isabs(_nvcc()) else "/usr/local/cuda"
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-fvisibility=hidden", "-shared",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           "-isystem", os.path.join(t, "include"), "-isystem", os.path.join(t, "include", "torch", "csrc", "api", "include"),
+           "-isystem", sysconfig.get_paths()["include"], "-isystem", os.path.join(cuda, "include"), NATIVE_SOURCE, "-o", NATIVE,
+           "-L", os.path.join(t, "lib"), "-ltorch_python", "-ltorch_cuda", "-ltorch_cpu", "-lc10_cuda", "-lc10"]
+    if verbose:
+        print(" ".join(cmd), flush=True)
+    subprocess.run(cmd, check=True)
+    return NATIVE
 
 
 def needs_build() -> bool:
@@ -71,6 +96,8 @@ def spill_report():
 def build(force: bool = False, verbose: bool = False, extra_flags=(), out: str = LIB) -> str:
     """Compiles every .cu of the library and links `out`.  `extra_flags` (for example -DMARLIN_TIMING)
     and a different `out` give an instrumented variant beside the product library."""
+    if out == LIB:
+        build_native(force, verbose)
     if not force and out == LIB and not needs_build():
         return LIB
     objs = []

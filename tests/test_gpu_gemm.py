@@ -387,3 +387,27 @@ def test_layer_object_makes_the_same_calls(marlin, oracle_lib):
         marlin.Layer(w, s, K, N, 64, ws)        # scale buffer does not match the group size
     with pytest.raises(ValueError):
         marlin.Layer(w, s, K, N, G, ws, max_M=100000)
+
+
+@pytest.mark.parametrize("bad,error", [
+    ("cpu", TypeError), ("dtype", TypeError), ("list", TypeError), ("strided", ValueError), ("wrong_k", ValueError),
+    ("one_dim", ValueError), ("out_rows", ValueError), ("out_dtype", TypeError), ("short_codes", ValueError)])
+def test_native_binding_refuses_what_the_kernels_cannot_take(marlin, bad, error):
+    import torch
+    case = inputs.make_dense(4, 256, 192, 128, seed=3)
+    layer = DenseLayer(marlin, case.q_kpacked, case.S, 128, max_M=4)
+    A, w, out = to_dev(case.A), layer.w, None
+    if bad == "cpu": A = A.cpu()
+    if bad == "dtype": A = A.float()
+    if bad == "list": A = [1.0]
+    if bad == "strided": A = to_dev(np.concatenate([case.A, case.A], axis=1))[:, ::2]
+    if bad == "wrong_k": A = A[:, :128].contiguous()
+    if bad == "one_dim": A = A[0]
+    if bad == "out_rows": out = torch.empty((5, 192), dtype=torch.float16, device="cuda")
+    if bad == "out_dtype": out = torch.empty((4, 192), dtype=torch.float32, device="cuda")
+    if bad == "short_codes": w = w[:-16]
+    with pytest.raises(error):
+        marlin.gemm(A, w, layer.s, 256, 192, 128, layer.ws, out=out)
+    if bad != "short_codes":
+        with pytest.raises((TypeError, ValueError)):
+            marlin.Layer(w, layer.s, 256, 192, 128, layer.ws)(A, out=out)
