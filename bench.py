@@ -767,7 +767,7 @@ def run_ours(args):
                                         "frac": round(step_achieved / peaks["hbm_gbs"], 4),
                                         "per_launch_us": round(step_s * 1e6 / launches_per_step, 3),
                                         "algorithmic_bytes_per_step": step_alg_bytes,
-                                        "kernels": "gemm_dense_kernel (M <= 16), gemm_dense_tc_kernel (M = 32, 64, 128)"}},
+                                        "kernels": "gemm_dense_kernel (M <= 16), gemm_tc_kernel (M = 32, 64, 128)"}},
             "per_m": per_m,
             "other_layers": extra,
             "cpu_baseline": {"value": round(cpu_v, 4), "unit": UNIT, "cores": cores, "kind": "oracle",

@@ -63,15 +63,6 @@ int tc_min_m() {
   return v;
 }
 
-// The tcgen05 kernel with deferred scales and 128-column tiles (gemm_tcd.cu) takes the layers whose N is a
-// multiple of 128 but not of 256 at batch sizes above 16.  MARLIN_B200_TCD (tuning knob): 0 switches it off
-// (slabs of 16 rows through the warp-level kernel instead), 1 makes it take every batch size on every layer
-// whose N is a multiple of 128 (64 rows per launch).
-int tcd_mode() {
-  const char* e = getenv("MARLIN_B200_TCD");  // read at every call, like the other tuning knobs
-  return !e ? 2 : (atoi(e) == 0 ? 0 : 1);     // 0 off, 1 everywhere, 2 default
-}
-
 }  // namespace
 
 extern "C" {
@@ -107,37 +98,19 @@ size_t marlin_packed_meta_bytes(int K, int N) {
   return (size_t)K * N / 8;
 }
 
-// Workspace map: [status word, counters: 8192 bytes][partial-tile slots of the warp-MMA kernel and of the tcgen05
-// kernel with deferred scales: a region of FIXED size][fp32 accumulation tiles of the tcgen05 kernel].
-// The counters and the accumulation tiles are zero at rest and every kernel leaves them that way; the slots are
-// written before they are read in every call and keep what the last call left.  Both boundaries are the same for
-// every layer, batch size and buffer size, so one buffer may serve calls on different layers one after the other:
-// the slots of one call never fall into the accumulation tiles of another.
-// two slots per worker, each the widest partial tile: 16 rows x 256 columns (warp-level kernel) or 64 rows x 128
-// columns (deferred scales)
-constexpr size_t kWsSlotFloats = (size_t)kWsSlotCols * kMaxSlabM > (size_t)128 * kTcdMaxSlabM ? (size_t)kWsSlotCols * kMaxSlabM
-                                                                                                : (size_t)128 * kTcdMaxSlabM;
-constexpr size_t kWsSlotRegionBytes = (size_t)2 * kMaxWorkers * kWsSlotFloats * sizeof(float);
-constexpr size_t kWsTcOff = kWsPartialOff + kWsSlotRegionBytes;
-// what the warp-level kernel alone needs: counters and its own slots
+// Workspace map: [status word, counters: 8192 bytes][partial-tile slots].  The counters are zero at rest and every kernel
+// leaves them that way; the slots are written before they are read in every call and keep what the last call left.
+// So one buffer may serve calls on different layers, batch sizes and formats one after the other.
+// What the warp-level kernel needs: two slots per worker of 16 rows x 256 columns.
 constexpr size_t kWarpOnlyWsBytes = kWsPartialOff + (size_t)2 * kMaxWorkers * kWsSlotCols * kMaxSlabM * sizeof(float);
-// sparse24: 2:4 layers on the wide layout run on the tcgen05 kernel at every batch size
-static size_t tc_tile_bytes(int max_M, int N, bool sparse24) {
-  if ((!sparse24 && max_M < tc_min_m()) || N % 256) return 0;
-  // one tile of 256 columns x padded rows per column tile; above 128 rows per worker at most (one launch takes all rows)
-  return tc_fixup_tiles(max_M, N, kMaxWorkers) * 256 * (size_t)tc_mpad(max_M < kTcMaxSlabM ? max_M : kTcMaxSlabM) *
-         sizeof(float);
-}
-static size_t workspace_bytes_for(int max_M, int K, int N, bool sparse24) {
-  (void)K;
-  return kWsTcOff + tc_tile_bytes(max_M, N, sparse24);
+static size_t workspace_bytes_for(int max_M, int K, int N) {
+  const size_t tc = kWsPartialOff + tc_slot_bytes(max_M, K, N);
+  return tc > kWarpOnlyWsBytes ? tc : kWarpOnlyWsBytes;
 }
 
 size_t marlin_workspace_bytes(int max_M, int K, int N) {
   if (max_M < 1 || !shape_ok(K, N)) return 0;
-  // the larger of what a dense and a 2:4 layer of this shape need (the query does not know which it will be)
-  const size_t d = workspace_bytes_for(max_M, K, N, false), sp = workspace_bytes_for(max_M, K, N, true);
-  return d > sp ? d : sp;
+  return workspace_bytes_for(max_M, K, N);
 }
 
 int marlin_pack(const uint32_t* q_kpacked, const void* scales, void* w_packed, void* s_packed, int K, int N,
@@ -212,8 +185,6 @@ static int gemm_common(const void* A, const void* w_packed, const void* meta_pac
                        bool sparse24, const void* z_packed = nullptr, bool swiglu = false, bool w8 = false,
                        bool warp_kernel_only = false) {
   if (!A || !w_packed || !s_packed || !C || !workspace || (sparse24 && !meta_packed)) return MARLIN_ERR_NULL;
-  // layers with zero points: the warp-level kernel up to 16 rows (and in slabs where N is not a multiple of 256), the
-  // tcgen05 kernel above
   const bool zero_points = z_packed != nullptr;
   if (zero_points && !aligned16(z_packed)) return MARLIN_ERR_ALIGN;
   if (w8 && N % 256) return MARLIN_ERR_SHAPE;  // 8-bit codes: the tcgen05 kernel alone, at every batch size
@@ -225,7 +196,7 @@ static int gemm_common(const void* A, const void* w_packed, const void* meta_pac
     return MARLIN_ERR_ALIGN;
   // (warp_kernel_only: the built-in array of marlin_gemm_static_ws, which holds the counters and the slots of the
   // warp-level kernel and nothing else; its caller has checked that this kernel serves the call)
-  if (workspace_bytes < (warp_kernel_only ? kWarpOnlyWsBytes : workspace_bytes_for(M, K, N, sparse24 || G < kTileK || zero_points || w8)))
+  if (workspace_bytes < (warp_kernel_only ? kWarpOnlyWsBytes : workspace_bytes_for(M, K, N)))
     return MARLIN_ERR_WORKSPACE;
   DeviceInfo info;
   int st = device_info(&info);
@@ -236,23 +207,14 @@ static int gemm_common(const void* A, const void* w_packed, const void* meta_pac
   int m0 = 0;
   while (m0 < M) {
     const int rem = M - m0;
-    // Which kernel takes the next rows.  Up to 16: the warp-level kernel.  Above: the tcgen05 kernel with
-    // in-loop scales (N a multiple of 256; all rows in one launch, slabs of 128 rows sharing its stripes), or the
-    // one with deferred scales (64 rows per launch, N a multiple of 128).  What none of them serves (2:4 layers, other N) goes through the warp-level
-    // kernel in slabs of 16 rows.
-    const int tmode = tcd_mode();
-    // 2:4 layers whose N is a multiple of 256 are packed in the wide layout, which only the tcgen05 kernel reads:
-    // it takes every batch size there
-    const bool tc_ok = tc_path_supported(1, K, N);
-    // groups of 64 or 32 rows likewise (accepted only where N is a multiple of 256)
-    const bool small_groups = G < kTileK || w8;
-    // (the kernel with deferred scales has no fused activation: those layers go through the warp-level kernel then)
-    const bool use_tcd = !warp_kernel_only && !swiglu && !sparse24 && !small_groups && !zero_points &&
-                         tcd_path_supported(1, K, N) && (tmode == 1 || (tmode == 2 && rem >= tc_min_m() && !tc_ok));
-    const bool use_tc = !warp_kernel_only && !use_tcd && tc_ok && (sparse24 || small_groups || rem >= tc_min_m());
-    const int m_slab = use_tcd ? (rem < kTcdMaxSlabM ? rem : kTcdMaxSlabM)
-                               : use_tc ? (rem < tc_max_rows(K, N, info.sm_count) ? rem : tc_max_rows(K, N, info.sm_count))
-                                        : (rem < kMaxSlabM ? rem : kMaxSlabM);
+    // Which kernel takes the next rows.  Up to 16: the warp-level kernel.  Above: the tcgen05 kernel, all rows in one
+    // launch.  2:4 layers whose N is a multiple of 256 are packed in the wide layout, which only the tcgen05 kernel
+    // reads: it takes every batch size there, and likewise groups of 64 or 32 rows and 8-bit codes (accepted only
+    // where N is a multiple of 256).  Other 2:4 layers go through the warp-level kernel in slabs of 16 rows.
+    const bool wide = N % 256 == 0;
+    const bool use_tc = !warp_kernel_only && (sparse24 ? wide : (G < kTileK || w8 || rem >= tc_min_m()));
+    const int max_rows = use_tc ? tc_max_rows(K, N, info.sm_count) : kMaxSlabM;
+    const int m_slab = rem < max_rows ? rem : max_rows;
     GemmParams p;
     p.A = static_cast<const uint16_t*>(A) + (size_t)m0 * K;
     p.wq = static_cast<const uint8_t*>(w_packed);
@@ -274,16 +236,13 @@ static int gemm_common(const void* A, const void* w_packed, const void* meta_pac
     p.status = reinterpret_cast<int*>(ws + kWsStatusOff);
     p.counters = reinterpret_cast<int*>(ws + kWsCounterOff);
     p.partials = reinterpret_cast<float*>(ws + kWsPartialOff);
-    p.tc_tiles = use_tc ? reinterpret_cast<float*>(ws + kWsTcOff) : nullptr;
     p.split = 0;
     p.whole = 0;
     p.slabs = 1;
     p.cluster = 0;
     p.slot_floats = kWsSlotCols * kMaxSlabM;
-    if (use_tcd) {
-      if (launch_gemm_tcd(p, info.sm_count, static_cast<cudaStream_t>(stream)) != cudaSuccess) return MARLIN_ERR_CUDA;
-    } else if (use_tc) {
-      if (launch_gemm_dense_tc(p, info.sm_count, sparse24, static_cast<cudaStream_t>(stream), w8) != cudaSuccess)
+    if (use_tc) {
+      if (launch_gemm_tc(p, info.sm_count, sparse24, w8, static_cast<cudaStream_t>(stream)) != cudaSuccess)
         return MARLIN_ERR_CUDA;
     } else {
       DensePlan plan;

@@ -26,8 +26,6 @@ constexpr int kProducerRegs = 40;
 constexpr int kMaxStages = 32;
 constexpr int kMaxWorkers = 160;      // grid size cap (a B200 has 148 SMs)
 constexpr int kMaxSlabM = 16;         // rows of A handled by one launch of the mma.sync kernel
-constexpr int kTcMaxSlabM = 128;      // rows of A handled by one launch of the tcgen05 kernel with in-loop scales
-constexpr int kTcdMaxSlabM = 64;      // rows of A handled by one launch of the tcgen05 kernel with deferred scales
 constexpr int kSmemBudget = 227 * 1024;
 
 // workspace layout (bytes)
@@ -76,14 +74,14 @@ struct GemmParams {
   int stage_bytes;
   int* status;
   int* counters;
-  float* partials;   // warp-MMA kernel: partial-tile slots
-  float* tc_tiles;   // tcgen05 kernel: one fp32 accumulation tile per 256-column tile
-  int slot_floats;   // floats per partial-tile slot
+  float* partials;   // partial-tile slots of the fix-up
+  int slot_floats;   // warp-MMA kernel: floats per slot
   int swiglu;        // 1: the columns come in blocks of 16 (eight gate channels, then the same eight up channels) and the
                      // kernel stores silu(gate) * up, N / 2 columns per row of C
-  uint32_t cluster;  // tcgen05 kernel: 1 = launched as thread-block clusters of `split` CTAs (the CTAs of one column tile)
-  uint32_t slabs;    // tcgen05 kernel: slabs of 128 batch rows in this launch (1 up to 128 rows); virtual column tile
-                     // v = column tile v / slabs of W, batch rows 128 * (v % slabs) ..
+  uint32_t cluster;  // warp-MMA kernel: 1, 2 = the CTAs of a column tile form a cluster (see there); tcgen05 kernel: CTAs per
+                     // cluster (a divisor of `split`; 0, 1: none)
+  uint32_t slabs;    // tcgen05 kernel: slabs of batch rows (32, 64 or 128) in this launch; virtual column tile
+                     // v = column tile v / slabs of W, rows of slab v % slabs
   uint32_t whole;    // tcgen05 kernel: 1 = worker w owns the virtual column tiles [w * ncols / P, (w + 1) * ncols / P) whole
   uint32_t split;    // tcgen05 kernel: 0 = even stripes over all units; S > 0 = every column tile is cut into S
                      // k-ranges and worker w owns range w % S of tile w / S (one segment per CTA)
@@ -93,23 +91,14 @@ cudaError_t launch_gemm_dense(const DensePlan& plan, const GemmParams& p, int fm
 cudaError_t launch_pack_sparse24(uint32_t* qc, uint8_t* idx, uint16_t* s, uint32_t* wq, uint32_t* meta, uint16_t* sq, int K,
                                  int N, int G, bool inverse, cudaStream_t stream);
 
-// tcgen05 kernel (gemm_dense_tc.cu): 256-column tiles, up to 128 rows of A per launch.
-bool tc_path_supported(int m_slab, int K, int N);
-int tc_mpad(int m_slab);  // rows of A padded to the MMA's N: 32, 64 or 128
-int tc_max_rows(int K, int N, int sm_count);      // most rows one launch takes (a multiple of 128)
-size_t tc_fixup_tiles(int M, int N, int workers); // fp32 accumulation tiles (256 columns x padded rows) the fix-up needs
-// fills the plan fields of `p` (ncols, units, workers) itself; sparse24: the 2:4 instances (tcgen05.mma.sp), which read
-// the wide 2:4 layout (N a multiple of 256)
-// w8: the instances for 8-bit codes (N a multiple of 256)
-cudaError_t launch_gemm_dense_tc(GemmParams p, int sm_count, bool sparse24, cudaStream_t stream, bool w8 = false);
+// tcgen05 kernel (gemm_tc.cuh)
+int tc_max_rows(int K, int N, int sm_count);     // most rows one launch takes (a multiple of 64)
+size_t tc_slot_bytes(int M, int K, int N);       // workspace slots of a call with M rows (any format)
+// fills the plan fields of `p` (ncols, units, workers, ...) itself; sparse24: the 2:4 instances (tcgen05.mma.sp), which read
+// the wide 2:4 layout (N a multiple of 256); w8: the instances for 8-bit codes (N a multiple of 256)
+cudaError_t launch_gemm_tc(GemmParams p, int sm_count, bool sparse24, bool w8, cudaStream_t stream);
 // 8-bit codes uint8 [K][N] <-> packed [N/256][K/128][8 vectors][256 columns][16 bytes]
 cudaError_t launch_pack_w8(uint8_t* q8, uint8_t* wq, int K, int N, bool inverse, cudaStream_t stream);
-// tcgen05 kernel with deferred scales (gemm_tcd.cu): 128-column tiles, up to 64 rows of A per launch.
-bool tcd_path_supported(int m_slab, int K, int N);
-int tcd_mpad(int m_slab);            // rows of A padded to the MMA's N: 16, 32 or 64
-size_t tcd_slot_floats(int m_slab);  // floats of one partial-tile slot of the fix-up
-// fills the plan fields of `p` (ncols, units, workers, slot_floats) itself
-cudaError_t launch_gemm_tcd(GemmParams p, int sm_count, cudaStream_t stream);
 // inverse == false: (q, s) canonical inputs -> (wq, sq) packed outputs; inverse == true: the other way round.
 cudaError_t launch_pack_dense(uint32_t* q, uint16_t* s, uint32_t* wq, uint16_t* sq, int K, int N, int G, bool inverse,
                               cudaStream_t stream);

@@ -1,0 +1,76 @@
+"""GPU parity of the tcgen05 kernel (gemm_tc.cuh) where its variants meet: column tiles of 128 and 256, the edges of the
+row paddings, narrow last tiles, deferred scales above 64 rows, both conversions, one and several clusters per tile.
+
+Bound: |C - C_ref| <= 5e-3 * (|C_ref| + rms(C_ref)) per element, the bound of the layer.
+"""
+import numpy as np
+import pytest
+
+from paper_2408_11743_b200 import inputs
+from gpu_util import DenseLayer, SparseLayer
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def marlin():
+    import torch
+    assert torch.cuda.is_available()
+    import paper_2408_11743_b200 as m
+    m.lib()
+    return m
+
+
+def _check(oracle_lib, C, C_ref):
+    bad, worst, rms = oracle_lib.check_tolerance(C, C_ref)
+    assert bad == 0, f"{bad} elements out of tolerance, worst ratio {worst:.3f}, rms {rms:.3f}"
+
+
+# rows at the edges of the paddings (32, 64, 128, slabs); N of whole tiles, of a narrow last one, of 64 columns alone
+@pytest.mark.parametrize("tile", ["128", "256"])
+@pytest.mark.parametrize("M,K,N,G", [(17, 128, 256, 128), (32, 384, 512, 128), (33, 512, 320, -1), (64, 1024, 256, 128),
+                                     (65, 640, 64, -1), (128, 2048, 768, 128), (129, 512, 1024, -1), (300, 256, 448, -1)])
+def test_both_tile_widths_match_the_oracle_and_are_reproducible(marlin, oracle_lib, monkeypatch, tile, M, K, N, G):
+    monkeypatch.setenv("MARLIN_B200_TC_TILE", tile)
+    case = inputs.make_dense(M, K, N, G, seed=M + K + N)
+    layer = DenseLayer(marlin, case.q_kpacked, case.S, case.G, max_M=M)
+    C = layer(case.A)
+    _check(oracle_lib, C, oracle_lib.gemm(case.A, case.q_kpacked, case.S, case.G))
+    assert np.array_equal(layer(case.A).view(np.uint16), C.view(np.uint16))  # partial tiles are added in a fixed order
+
+
+# deferred scales: N a multiple of 64 but not of 256
+@pytest.mark.parametrize("M", [17, 33, 64, 65, 128, 129, 300])
+@pytest.mark.parametrize("K,N,G", [(256, 64, 128), (1152, 448, 384), (2048, 1344, 128)])
+def test_deferred_scales_at_every_row_padding(marlin, oracle_lib, M, K, N, G):
+    case = inputs.make_dense(M, K, N, G, seed=M + K + N)
+    C = DenseLayer(marlin, case.q_kpacked, case.S, G, max_M=M)(case.A)
+    _check(oracle_lib, C, oracle_lib.gemm(case.A, case.q_kpacked, case.S, G))
+
+
+# few column tiles and a long K: several clusters share a tile, their shares meet in the workspace
+@pytest.mark.parametrize("M,K,N,G", [(20, 16384, 256, 128), (128, 16384, 512, 128), (48, 8192, 192, 128), (100, 12288, 320, -1)])
+def test_several_clusters_per_tile(marlin, oracle_lib, M, K, N, G):
+    case = inputs.make_dense(M, K, N, G, seed=M + N)
+    layer = DenseLayer(marlin, case.q_kpacked, case.S, case.G, max_M=M)
+    C = layer(case.A)
+    _check(oracle_lib, C, oracle_lib.gemm(case.A, case.q_kpacked, case.S, case.G))
+    assert np.array_equal(layer(case.A).view(np.uint16), C.view(np.uint16))
+
+
+# the conversion with one fma per pair holds for scales up to 0.0624; larger, negative and zero ones among them
+@pytest.mark.parametrize("sparse", [False, True])
+@pytest.mark.parametrize("G", [128, 64, 32])
+def test_scales_on_both_sides_of_the_short_conversion(marlin, oracle_lib, sparse, G):
+    M, K, N = 40, 1024, 512
+    case = (inputs.make_sparse24 if sparse else inputs.make_dense)(M, K, N, G, seed=G)
+    rng = np.random.default_rng(G)
+    S = case.S.copy()
+    S[:, : N // 2] *= rng.choice(np.array([1, -1, 3, 40, 0], np.float16), size=(S.shape[0], N // 2))
+    S[0, :4] = [0.0624, 0.0625, 0.06238, -0.0625]  # the last fp16 values on either side
+    case.S = S
+    if sparse:
+        _check(oracle_lib, SparseLayer(marlin, case, M)(case.A),
+               oracle_lib.gemm_sparse24(case.A, case.qc_kpacked, case.idx, S, G))
+    else:
+        _check(oracle_lib, DenseLayer(marlin, case.q_kpacked, S, G, max_M=M)(case.A), oracle_lib.gemm(case.A, case.q_kpacked, S, G))
