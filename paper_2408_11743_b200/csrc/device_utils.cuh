@@ -108,16 +108,7 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
       ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)), "l"(pol)
       : "memory");
 }
-// One box of a 2-D tensor map -> shared memory (no multicast: every CTA fetches its own copy).
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y, uint64_t* bar,
-                                            uint64_t pol) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
-      " [%0], [%1, {%2, %3}], [%4], %5;"
-      ::"r"(smem_u32(dst)), "l"(map), "r"(x), "r"(y), "r"(smem_u32(bar)), "l"(pol)
-      : "memory");
-}
-// One box of a 3-D tensor map -> shared memory
+// One box of a 3-D tensor map -> shared memory (no multicast: every CTA fetches its own copy).
 __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, int x, int y, int z, uint64_t* bar,
                                             uint64_t pol) {
   asm volatile(
@@ -300,7 +291,6 @@ __device__ __forceinline__ void pdl_wait_prior_grids() { asm volatile("griddepco
 __device__ __forceinline__ float4 ld_cg_f4(const float4* p) { return __ldcg(p); }
 
 // tensor maps are built through the runtime's driver entry point (no link against libcuda)
-bool make_a_tensor_map(CUtensorMap* map, const void* A, int M, int K, int box_rows);
 // A[M][K] as a 3-D tensor (64 columns, M rows, K / 64 column blocks): one box of 64 x box_rows x 2 brings both
 // 64-wide halves of a 128-row k-block, each as a 128-byte-swizzled tile of box_rows rows, one after the other
 bool make_a_tensor_map_3d(CUtensorMap* map, const void* A, int M, int K, int box_rows);
