@@ -237,6 +237,8 @@ static int gemm_common(const void* A, const void* w_packed, const void* meta_pac
     p.counters = reinterpret_cast<int*>(ws + kWsCounterOff);
     p.partials = reinterpret_cast<float*>(ws + kWsPartialOff);
     p.split = 0;
+    p.team_tiles = 0;
+    p.team_extra = 0;
     p.whole = 0;
     p.slabs = 1;
     p.cluster = 0;
@@ -252,6 +254,8 @@ static int gemm_common(const void* A, const void* w_packed, const void* meta_pac
       p.units = (uint32_t)plan.units;
       p.workers = (uint32_t)plan.workers;
       p.split = (uint32_t)plan.split;
+      p.team_tiles = (uint32_t)(plan.ncols / plan.teams);
+      p.team_extra = (uint32_t)(plan.ncols % plan.teams);
       p.stages = plan.stages;
       p.stage_bytes = plan.stage_bytes;
       if (launch_gemm_dense(plan, p, fmt, static_cast<cudaStream_t>(stream)) != cudaSuccess) return MARLIN_ERR_CUDA;
@@ -439,7 +443,7 @@ int marlin_plan_stripes(int M, int K, int N, int sm_count, int* n_tile, int* wor
   if (M < 1 || !shape_ok(K, N)) return MARLIN_ERR_SHAPE;
   DensePlan plan;
   const int m_slab = M < kMaxSlabM ? M : kMaxSlabM;
-  if (!make_dense_plan(m_slab, K, N, sm_count, false, &plan)) return MARLIN_ERR_SHAPE;
+  if (!make_dense_plan(m_slab, K, N, sm_count, false, &plan, false)) return MARLIN_ERR_SHAPE;
   if (cap < plan.workers + 1) return MARLIN_ERR_SHAPE;
   *n_tile = plan.nw * kChunkN;
   *workers = plan.workers;

@@ -137,9 +137,20 @@ gemm_dense_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a
   const int lane = threadIdx.x & 31;
   const uint32_t worker = blockIdx.x;
   const uint32_t U = p.units, P = p.workers, KB = p.kb;
-  // split > 0: one k-range of one column tile per CTA instead of an even stripe over all units
-  const uint32_t u0 = p.split ? split_begin32(worker, KB, p.split) : stripe_begin32(worker, U, P);
-  const uint32_t u1 = p.split ? split_begin32(worker + 1, KB, p.split) : stripe_begin32(worker + 1, U, P);
+  // split > 0: teams of `split` CTAs share consecutive column tiles evenly, instead of an even stripe over all units
+  // (few divisions: the first copies wait for the result)
+  uint32_t u0, u1, team = 0, team_c0 = 0, team_units = 0;
+  if (p.split) {
+    team = worker / p.split;
+    const uint32_t rank = worker - team * p.split;
+    team_c0 = team_first_tile(team, p.team_tiles, p.team_extra);
+    team_units = (team_first_tile(team + 1, p.team_tiles, p.team_extra) - team_c0) * KB;
+    u0 = team_c0 * KB + rank * team_units / p.split;
+    u1 = team_c0 * KB + (rank + 1) * team_units / p.split;
+  } else {
+    u0 = stripe_begin32(worker, U, P);
+    u1 = stripe_begin32(worker + 1, U, P);
+  }
   const int nstages = p.stages;
 
   pdl_launch_dependents();
@@ -162,6 +173,12 @@ gemm_dense_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a
     asm volatile("bar.arrive 3, %0;" ::"n"((CW + 4) * 32) : "memory");
   } else {
     asm volatile("bar.sync 3, %0;" ::"n"((CW + 4) * 32) : "memory");
+  }
+  // Teams with several column tiles write to another CTA's shared memory early: the wait for this arrival, before the first
+  // such write, makes sure that it has started.
+  if (p.cluster == 3) {
+    __syncwarp();
+    cluster_arrive();
   }
 
   if (warp >= kConsumerWarps) {
@@ -256,6 +273,8 @@ gemm_dense_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a
     }
     if (p.cluster) {
       // every thread of every CTA of the cluster takes part in the barriers of the fix-up
+      __syncwarp();
+      if (p.cluster == 3) cluster_wait();
       if (p.cluster == 1) cluster_sync_all();
       cluster_sync_all();
     }
@@ -356,6 +375,14 @@ gemm_dense_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a
     }
   };
 
+  // the workspace slot in which worker w left its part of a tile
+  auto slot_of = [&](int w, uint32_t col) {
+    if (p.split && team_units == KB) return 2 * w;
+    const uint32_t begin = p.split ? team_c0 * KB + (uint32_t)(w - (int)(team * p.split)) * team_units / p.split
+                                   : stripe_begin32((uint32_t)w, U, P);
+    return 2 * w + (col != begin / KB ? 1 : 0);
+  };
+  bool team_started = p.cluster != 3;
   uint32_t u = u0;
   uint32_t it0 = 0;  // iteration index of the segment's first unit, relative to u0
   while (u < u1) {
@@ -549,14 +576,40 @@ gemm_dense_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a
     named_bar_sync(1, kConsumerThreads);  // `red` may be written again
 
     // ---- stripe fix-up across CTAs and output ----
-    const int first_w = p.split ? (int)(col * p.split) : (int)stripe_owner32(col * KB, U, P);
-    const int last_w = p.split ? (int)(col * p.split + p.split - 1) : (int)stripe_owner32((col + 1) * KB - 1, U, P);
+    const int team_w = (int)(team * p.split);  // the first CTA of the team
+    int first_w, last_w;                        // the CTAs that share the tile
+    if (p.split && team_units == KB) {
+      first_w = team_w;
+      last_w = team_w + (int)p.split - 1;
+    } else if (p.split) {
+      first_w = team_w + (int)stripe_owner32((col - team_c0) * KB, team_units, p.split);
+      last_w = team_w + (int)stripe_owner32((col - team_c0 + 1) * KB - 1, team_units, p.split);
+    } else {
+      first_w = (int)stripe_owner32(col * KB, U, P);
+      last_w = (int)stripe_owner32((col + 1) * KB - 1, U, P);
+    }
+    // Clusters: the partial tiles go to the shared memory of the tile's first CTA (for which the tile is its last segment: it
+    // receives those of one tile only), behind its ring or into it
+    const uint32_t xbuf = p.cluster >= 2 ? stage0_s + (uint32_t)nstages * G::STAGE_BYTES : stage0_s;
+    auto wait_for_team = [&]() {
+      if (!team_started) cluster_wait();
+      team_started = true;
+    };
+    auto send_partial = [&]() {
+      wait_for_team();
+      const uint32_t dst = xbuf + (uint32_t)((((int)worker - first_w - 1) * G::TILE_F4 + wn * G::FRAG_F4 * 32 + lane) * 16);
+#pragma unroll
+      for (int r = 0; r < 4 * MB; ++r)
+        st_cluster_f32x4(dst + (uint32_t)(r * 32 * 16), (uint32_t)(first_w - team_w), acc[r][0], acc[r][1], acc[r][2], acc[r][3]);
+    };
     if (u + len < u1) {
       // A segment in the middle of the stripe: group 0 holds the tile and finishes it alone (its L2 round
       // trips take a microsecond or two); the other groups go on with the k-blocks of the next segment.
       if (grp == 0) {
         constexpr int kG0 = NW * 32;
-        if (last_w > first_w) {
+        if (last_w > first_w && p.cluster) {
+          send_partial();  // (never the tile's first CTA: that one's part of a shared tile ends its stripe)
+        } else if (last_w > first_w) {
           const int my_slot = 2 * (int)worker + (col != u0 / KB ? 1 : 0);
           float4* mine = reinterpret_cast<float4*>(p.partials + (size_t)my_slot * p.slot_floats) +
                          (size_t)wn * G::FRAG_F4 * 32 + lane;
@@ -573,7 +626,7 @@ gemm_dense_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a
           if (last_flag[1]) {
             // every thread re-reads its own fragment positions of all partials, in stripe order
             for (int w = first_w; w <= last_w; ++w) {
-              const int slot = 2 * w + ((!p.split && col != stripe_begin32(w, U, P) / KB) ? 1 : 0);
+              const int slot = slot_of(w, col);
               const float4* src = reinterpret_cast<const float4*>(p.partials + (size_t)slot * p.slot_floats) +
                                   (size_t)wn * G::FRAG_F4 * 32 + lane;
 #pragma unroll
@@ -588,7 +641,7 @@ gemm_dense_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a
             }
           }
         }
-        if (last_w == first_w || last_flag[1]) {
+        if (last_w == first_w || (!p.cluster && last_flag[1])) {
 #pragma unroll
           for (int r = 0; r < 4 * MB; ++r) {
             const int j = r / MB, mb = r % MB;
@@ -611,19 +664,15 @@ gemm_dense_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a
     // ---- the last segment of the stripe: all consumer threads take part ----
     bool tile_in_cst = false;
     if (p.cluster) {
-      // The CTAs of this column tile form a thread-block cluster and finish side by side.  The partial tiles
-      // go straight into the shared memory of the cluster's first CTA (its stage ring is free by now), which
+      // The CTAs of a team form a thread-block cluster and finish side by side.  The partial tiles
+      // go straight into the shared memory of the tile's first CTA, which
       // adds them to its own in rank order: the order of the workspace path, without its L2 round trips.
-      // (cluster == 2: the launch has room for the partial tiles behind the stage ring, which nobody else touches:
+      // (cluster >= 2: the launch has room for the partial tiles behind the stage ring, which nobody else touches:
       // no need to wait until the first CTA is done with its ring)
       const int rank = (int)worker - first_w;
-      const uint32_t xbuf = p.cluster == 2 ? stage0_s + (uint32_t)nstages * G::STAGE_BYTES : stage0_s;
       if (p.cluster == 1) cluster_sync_all();  // every CTA of the tile is done with its stage ring
-      if (rank != 0 && grp == 0) {
-        const uint32_t dst = xbuf + (uint32_t)(((rank - 1) * G::TILE_F4 + wn * G::FRAG_F4 * 32 + lane) * 16);
-#pragma unroll
-        for (int r = 0; r < 4 * MB; ++r) st_cluster_f32x4(dst + (uint32_t)(r * 32 * 16), 0u, acc[r][0], acc[r][1], acc[r][2], acc[r][3]);
-      }
+      if (rank != 0 && grp == 0) send_partial();
+      wait_for_team();
       cluster_sync_all();  // the partial tiles have arrived
       if (rank == 0) {
         if (grp == 0) {
@@ -679,7 +728,7 @@ gemm_dense_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a
           for (int d = 0; d < BATCH; ++d) {
             const int ww = w + d;
             if (ww <= last_w) {
-              const int slot = 2 * ww + ((!p.split && col != stripe_begin32(ww, U, P) / KB) ? 1 : 0);
+              const int slot = slot_of(ww, col);
               const float4* src = reinterpret_cast<const float4*>(p.partials + (size_t)slot * p.slot_floats);
 #pragma unroll
               for (int e = 0; e < PER; ++e) {
@@ -811,8 +860,13 @@ cudaError_t launch_one(const DensePlan& plan, const GemmParams& p, cudaStream_t 
   q.cluster = 0;
   const int S = plan.split;
   const char* e = getenv("MARLIN_B200_CLUSTER");  // tuning knob: 0 = fix-up through the workspace
-  if (S >= 2 && S <= 8 && (size_t)(S - 1) * G_TILE_BYTES <= (size_t)plan.stages * plan.stage_bytes && !(e && atoi(e) == 0)) {
-    // the S CTAs of a column tile as one thread-block cluster, if all clusters of the grid fit on the device
+  // room behind the ring for the S - 1 partial tiles: the exchange then needs one cluster barrier instead of two; teams with
+  // several column tiles, whose partial tiles may come early, need it
+  const char* x = getenv("MARLIN_B200_XBUF");  // tuning knob: 0 = partial tiles into the first CTA's ring
+  const bool room = (size_t)plan.smem_bytes + (size_t)(S - 1) * G_TILE_BYTES <= (size_t)kSmemBudget && !(x && atoi(x) == 0);
+  const bool fits = room || (plan.teams == plan.ncols && (size_t)(S - 1) * G_TILE_BYTES <= (size_t)plan.stages * plan.stage_bytes);
+  if (S >= 2 && S <= 8 && fits && !(e && atoi(e) == 0)) {
+    // the S CTAs of a team as one thread-block cluster, if all clusters of the grid fit on the device
     // at once (a GPC holds only so many clusters of a size; a second wave would cost more than it saves)
     static int max_clusters[64][9] = {};  // per device and cluster size: clusters resident at once (0 unknown, -1 none)
     int nmax = (dev >= 0 && dev < 64) ? max_clusters[dev][S] : 0;
@@ -830,11 +884,9 @@ cudaError_t launch_one(const DensePlan& plan, const GemmParams& p, cudaStream_t 
     const int ok = (nmax > 0 && (long long)nmax * S >= plan.workers) ? 1 : -1;  // all clusters of THIS grid at once
     cfg.numAttrs = ok > 0 ? 2 : 1;
     q.cluster = ok > 0 ? 1u : 0u;
-    // room behind the ring for the S - 1 partial tiles: the exchange then needs one cluster barrier instead of two
-    const char* x = getenv("MARLIN_B200_XBUF");  // tuning knob: 0 = partial tiles into the first CTA's ring
-    if (ok > 0 && (size_t)plan.smem_bytes + (size_t)(S - 1) * G_TILE_BYTES <= (size_t)kSmemBudget && !(x && atoi(x) == 0)) {
+    if (ok > 0 && room) {
       cfg.dynamicSmemBytes = plan.smem_bytes + (S - 1) * G_TILE_BYTES;
-      q.cluster = 2u;
+      q.cluster = plan.teams < plan.ncols ? 3u : 2u;
     }
   }
   return cudaLaunchKernelEx(&cfg, kernel, q, tmap);
@@ -859,6 +911,9 @@ void fill_geometry(DensePlan* plan) {
                                                             : G::SK * kProducerWarps / (G::SK % 2 == 0 ? 2 : 1);
   static_assert(kRingUnit % G::SK == 0 && kRingUnit % kProducerWarps == 0, "ring unit must be a common multiple");
   stages -= stages % kRingUnit;
+  if (plan->teams < plan->ncols)  // room for the partial tiles that a team exchanges (see launch_one)
+    while (stages > kRingUnit && G::FIXED_BYTES + G::ALIGN_SLACK + stages * G::STAGE_BYTES + (plan->split - 1) * G::TILE_F4 * 16 > kSmemBudget)
+      stages -= kRingUnit;
   plan->stages = stages;
   plan->smem_bytes = G::FIXED_BYTES + G::ALIGN_SLACK + stages * G::STAGE_BYTES;
 }
@@ -880,7 +935,7 @@ cudaError_t launch_one_fmt(int fmt, const DensePlan& plan, const GemmParams& p, 
 }  // namespace
 
 
-bool make_dense_plan(int m_slab, int K, int N, int sm_count, int fmt, DensePlan* plan) {
+bool make_dense_plan(int m_slab, int K, int N, int sm_count, int fmt, DensePlan* plan, bool teams_too) {
   if (m_slab < 1 || m_slab > kMaxSlabM || K < kTileK || K % kTileK || N < kChunkN || N % kChunkN) return false;
   if (sm_count < 1) return false;
   int mb = m_slab <= 8 ? 1 : 2;
@@ -925,6 +980,8 @@ bool make_dense_plan(int m_slab, int K, int N, int sm_count, int fmt, DensePlan*
   const long long even_n = (even_units + even_workers - 1) / even_workers;
   double best = base_us + even_us + chunk_us(even_nw, even_n) * (double)(even_n * even_nw);
   int nw = even_nw, split = 0;
+  // The stripes of the paper or the tile-aligned form, with the most CTAs; what a launch takes in their place comes below.
+  long long teams = 0;
   for (int cand = 1; cand <= 4 && allow_split; cand *= 2) {
     if (forced_nw && cand != forced_nw) continue;
     if (N % (kChunkN * cand)) continue;
@@ -935,7 +992,40 @@ bool make_dense_plan(int m_slab, int K, int N, int sm_count, int fmt, DensePlan*
     const long long stages_per_cta = (kb + S - 1) / S;
     if (mb != 1 && cand == 4 && S > 1 && !forced_nw) continue;
     const double cost = base_us + chunk_us(cand, stages_per_cta) * (double)(stages_per_cta * cand) + fixup_us(cand, S);
-    if (cost < best) { nw = cand; split = (int)S; best = cost; }
+    if (cost < best) { nw = cand; split = (int)S; teams = ncols; best = cost; }
+  }
+  // Teams of S CTAs, each with consecutive column tiles of its own: one tile (tile-aligned: any S), or several, cut evenly
+  // between two CTAs (whole tiles for S = 1), where no number of k-ranges uses the SMs well.  With more than two CTAs per
+  // team several tiles gain as much in a chain of equal launches, but clusters of three behind clusters of four leave SMs in
+  // pieces that the next ones do not fit: a wave more (gate_up 22016 columns, then down, one row: 29.9 us against 20.4 with
+  // pairs and 21.7 with even stripes).
+  // A grid of at most half of the SMs lets the next launch start beside it: 8192 x 1024 at one row 5.5 us with nine k-ranges,
+  // 4.1 with four (64 CTAs); 1024 x 1024 4.6 with eight, 3.0 with two.  Clusters of seven and eight start late.  Clusters that
+  // do not fit at once (`resident`: what the occupancy query returns on a B200) exchange through the workspace.
+  static const int resident[9] = {0, 148, 74, 45, 33, 26, 22, 15, 15};
+  if (teams_too && allow_split) {
+    double best_us = base_us + even_us + chunk_us(even_nw, even_n) * (double)(even_n * even_nw);
+    nw = even_nw;
+    split = 0;
+    for (int cand = 1; cand <= 4; cand *= 2) {
+      if (forced_nw && cand != forced_nw) continue;
+      if (N % (kChunkN * cand)) continue;
+      const long long ncols = N / (kChunkN * cand);
+      for (long long S = 1; S <= kb && S <= max_workers; ++S) {
+        if (S > 2 && S * ncols > max_workers) break;
+        const long long per = max_workers / S, T = (ncols + per - 1) / per;  // column tiles of a team
+        const long long C = (ncols + T - 1) / T;
+        const long long stages_per_cta = (T * kb + S - 1) / S;
+        if (mb != 1 && cand == 4 && S > 1 && !forced_nw) continue;
+        double cost = base_us + chunk_us(cand, stages_per_cta) * (double)(stages_per_cta * cand) + fixup_us(cand, S);
+        if (T > 1) cost += (mb == 1 ? 0.5 : 0.65) + 0.25 * (double)T;
+        if (mb == 1 && cand == 4 && S > 1) cost += 0.47;
+        if (S > 1 && S <= 8 && C > resident[S]) cost += 1.5;
+        if (2 * S * C <= max_workers) cost -= mb == 1 ? 0.75 : 0.5;
+        else if (S >= 7 && S <= 8) cost += mb == 1 ? 0.5 : 0.25;
+        if (cost < best_us) { nw = cand; split = (int)S; teams = C; best_us = cost; }
+      }
+    }
   }
   plan->mb = mb;
   plan->nw = nw;
@@ -943,7 +1033,8 @@ bool make_dense_plan(int m_slab, int K, int N, int sm_count, int fmt, DensePlan*
   plan->ncols = N / (kChunkN * nw);
   plan->units = (long long)plan->ncols * plan->kb;
   plan->split = split;
-  long long workers = split ? (long long)split * plan->ncols : max_workers;
+  plan->teams = split ? (int)teams : plan->ncols;
+  long long workers = split ? (long long)split * teams : max_workers;
   if (workers > plan->units) workers = plan->units;
   plan->workers = (int)workers;
   // Consumer warps: twelve for 128-column tiles (nw = 2) from 16 stages per CTA on.  Measured on B200 over 42 layer
@@ -953,7 +1044,7 @@ bool make_dense_plan(int m_slab, int K, int N, int sm_count, int fmt, DensePlan*
   // difference; the 2:4 instance gains nothing.
   int cw = consumer_warps_for(mb);
   if (mb == 1) {
-    const long long n = split ? (kb + split - 1) / split : (plan->units + workers - 1) / workers;
+    const long long n = (plan->units + workers - 1) / workers;
     if (want_cw == kWideConsumerWarps || (want_cw != consumer_warps_for(mb) && wide_pays(nw, n))) cw = kWideConsumerWarps;
   }
   for (;;) {

@@ -43,7 +43,8 @@ struct DensePlan {
   int ncols;       // N / (64 * nw)
   long long units; // ncols * kb
   int workers;     // CTAs
-  int split;       // 0: even stripes; S > 0: S k-ranges per column tile, one per CTA
+  int split;       // 0: even stripes over all units; S > 0: teams of S CTAs, each with consecutive column tiles of its own
+  int teams;       // number of teams (ncols: a column tile each, cut into S k-ranges)
   int stages;
   int stage_bytes;
   int smem_bytes;
@@ -52,7 +53,8 @@ struct DensePlan {
 // Chooses tile width, worker count and pipeline depth for one slab of m_slab <= 32 rows.
 // Pure host arithmetic.  Returns false on an unsupported shape.
 // fmt: 0 dense, 1 the 2:4 variant, 2 dense with zero points (the stage then carries a zero-point row)
-bool make_dense_plan(int m_slab, int K, int N, int sm_count, int fmt, DensePlan* plan);
+// teams_too: what a launch takes (teams of any form); otherwise the best of even stripes and of one column tile per team
+bool make_dense_plan(int m_slab, int K, int N, int sm_count, int fmt, DensePlan* plan, bool teams_too = true);
 
 struct GemmParams {
   const uint16_t* A;
@@ -78,7 +80,8 @@ struct GemmParams {
   int slot_floats;   // warp-MMA kernel: floats per slot
   int swiglu;        // 1: the columns come in blocks of 16 (eight gate channels, then the same eight up channels) and the
                      // kernel stores silu(gate) * up, N / 2 columns per row of C
-  uint32_t cluster;  // warp-MMA kernel: 1, 2 = the CTAs of a column tile form a cluster (see there); tcgen05 kernel: CTAs per
+  uint32_t team_tiles, team_extra;  // warp-MMA kernel, split > 0: column tiles per team; teams with one more
+  uint32_t cluster;  // warp-MMA kernel: 1, 2, 3 = the CTAs of a team form a cluster (see there); tcgen05 kernel: CTAs per
                      // cluster (a divisor of `split`; 0, 1: none)
   uint32_t slabs;    // tcgen05 kernel: slabs of batch rows (32, 64 or 128) in this launch; virtual column tile
                      // v = column tile v / slabs of W, rows of slab v % slabs
@@ -127,6 +130,13 @@ __device__ inline uint32_t stripe_owner32(uint32_t x, uint32_t U, uint32_t P) { 
 __device__ inline uint32_t split_begin32(uint32_t w, uint32_t KB, uint32_t S) {
   const uint32_t t = w / S, r = w - t * S;
   return t * KB + (r * KB) / S;
+}
+
+// Teams of S workers, C of them (warp-level kernel): the first ncols % C teams own ncols / C + 1 column tiles, the others
+// ncols / C, one team after the other; the workers of a team have even stripes over its k-blocks.  With C = ncols this is the
+// tile-aligned variant above.
+__host__ __device__ inline uint32_t team_first_tile(uint32_t t, uint32_t tiles, uint32_t extra) {
+  return t * tiles + (t < extra ? t : extra);
 }
 
 }  // namespace marlin_b200

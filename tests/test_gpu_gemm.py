@@ -411,3 +411,22 @@ def test_native_binding_refuses_what_the_kernels_cannot_take(marlin, bad, error)
     if bad != "short_codes":
         with pytest.raises((TypeError, ValueError)):
             marlin.Layer(w, layer.s, 256, 192, 128, layer.ws)(A, out=out)
+
+
+# teams of CTAs with several column tiles each: one and two CTAs, 64- and 128-column tiles, teams of unequal size, both block
+# counts, exchange through clusters and through the workspace
+@pytest.mark.parametrize("M,K,N,mode", [
+    (1, 256, 64 * 149, {}), (8, 256, 64 * 149, {"MARLIN_B200_NW": "1"}), (16, 384, 128 * 150, {"MARLIN_B200_NW": "2"}),
+    (3, 1280, 64 * 222, {"MARLIN_B200_NW": "1"}), (9, 1152, 128 * 172, {"MARLIN_B200_NW": "2"}),
+    (5, 4096, 22016, {}), (16, 4096, 22016, {}), (5, 4096, 22016, {"MARLIN_B200_CLUSTER": "0"}),
+    (16, 4096, 22016, {"MARLIN_B200_XBUF": "0"}), (8, 2048, 1024, {}), (2, 28672, 1024, {}),
+])
+def test_teams_with_several_column_tiles_match_oracle(marlin, oracle_lib, monkeypatch, M, K, N, mode):
+    for k, v in mode.items():
+        monkeypatch.setenv(k, v)
+    case = inputs.make_dense(M, K, N, 128, seed=77 + M + N)
+    layer = DenseLayer(marlin, case.q_kpacked, case.S, 128, max_M=M)
+    C_ref = oracle_lib.gemm(case.A, case.q_kpacked, case.S, 128)
+    C = layer(case.A)
+    _assert_close(oracle_lib, C, C_ref)
+    assert np.array_equal(C.view(np.uint16), layer(case.A).view(np.uint16))
