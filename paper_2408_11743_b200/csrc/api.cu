@@ -52,15 +52,22 @@ int device_info(DeviceInfo* out) {
   return MARLIN_OK;
 }
 
-// Batch size from which the tcgen05 kernel takes over from the warp-level MMA kernel.
-int tc_min_m() {
+// Batch size from which the tcgen05 kernel takes over from the warp-level MMA kernel.  17 rows (the warp-level kernel takes 16),
+// but nine for dense layers of more than 2^26 weights with one scale per column.  There both kernels multiply exact integers and
+// scale the fp32 sums, and the loop, not the start, decides: the warp-level kernel spends two MMAs per 16 x 16 weights from nine
+// rows on.  Measured on B200 at 16 rows, warp-level / tcgen05: 28672 x 8192 30.5 / 24.9 us, 4096 x 22016 16.1 / 15.2,
+// 8192 x 10240 14.9 / 13.1, 5120 x 13824 12.5 / 11.8, but 8192 x 8192 11.7 / 11.9, 4096 x 12288 10.3 / 10.6; 28672 x 8192 at eight
+// rows 22.5 / 25.1.  With group scales the tcgen05 kernel would need an accumulator per group (deferred scales) to be as
+// exact: 28672 x 8192 at 16 rows 32.5 / 40.6.
+int tc_min_m(int K, int N, bool one_scale) {
   static int v = -1;
   if (v < 0) {
-    const char* e = getenv("MARLIN_B200_TC_MIN_M");  // tuning knob; default below
-    v = e ? atoi(e) : 17;
-    if (v < 1) v = 1;
+    const char* e = getenv("MARLIN_B200_TC_MIN_M");  // tuning knob; 0: the rule above
+    v = e ? atoi(e) : 0;
+    if (v < 0) v = 0;
   }
-  return v;
+  if (v > 0) return v;
+  return one_scale && (long long)K * N > (1ll << 26) ? 9 : 17;
 }
 
 }  // namespace
@@ -207,12 +214,12 @@ static int gemm_common(const void* A, const void* w_packed, const void* meta_pac
   int m0 = 0;
   while (m0 < M) {
     const int rem = M - m0;
-    // Which kernel takes the next rows.  Up to 16: the warp-level kernel.  Above: the tcgen05 kernel, all rows in one
-    // launch.  2:4 layers whose N is a multiple of 256 are packed in the wide layout, which only the tcgen05 kernel
+    // Which kernel takes the next rows.  Up to 16 (tc_min_m): the warp-level kernel.  Above: the tcgen05 kernel, all rows
+    // in one launch.  2:4 layers whose N is a multiple of 256 are packed in the wide layout, which only the tcgen05 kernel
     // reads: it takes every batch size there, and likewise groups of 64 or 32 rows and 8-bit codes (accepted only
     // where N is a multiple of 256).  Other 2:4 layers go through the warp-level kernel in slabs of 16 rows.
     const bool wide = N % 256 == 0;
-    const bool use_tc = !warp_kernel_only && (sparse24 ? wide : (G < kTileK || w8 || rem >= tc_min_m()));
+    const bool use_tc = !warp_kernel_only && (sparse24 ? wide : (G < kTileK || w8 || rem >= tc_min_m(K, N, G == K && !zero_points)));
     const int max_rows = use_tc ? tc_max_rows(K, N, info.sm_count) : kMaxSlabM;
     const int m_slab = rem < max_rows ? rem : max_rows;
     GemmParams p;

@@ -74,3 +74,14 @@ def test_scales_on_both_sides_of_the_short_conversion(marlin, oracle_lib, sparse
                oracle_lib.gemm_sparse24(case.A, case.qc_kpacked, case.idx, S, G))
     else:
         _check(oracle_lib, DenseLayer(marlin, case.q_kpacked, S, G, max_M=M)(case.A), oracle_lib.gemm(case.A, case.q_kpacked, S, G))
+
+
+# one scale per column on a large layer: the rows at which the two kernels change over, on either side of the size rule
+@pytest.mark.parametrize("M", [8, 9, 16, 17])
+@pytest.mark.parametrize("K,N", [(8192, 8192), (8192, 8256), (3072, 22016)])
+def test_large_layers_with_one_scale_per_column_change_kernels_at_nine_rows(marlin, oracle_lib, M, K, N):
+    case = inputs.make_dense(M, K, N, -1, seed=5 + M + N)
+    layer = DenseLayer(marlin, case.q_kpacked, case.S, case.G, max_M=M)
+    C = layer(case.A)
+    bad, worst, rms = oracle_lib.check_tolerance(C, oracle_lib.gemm(case.A, case.q_kpacked, case.S, case.G))
+    assert bad == 0, (bad, worst, rms)
