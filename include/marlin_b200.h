@@ -66,10 +66,9 @@ MARLIN_API size_t marlin_packed_scale_bytes(int K, int N, int group_size);
 /* Bytes of the packed 2:4 metadata buffer: K*N/8 (2 bits per kept value). */
 MARLIN_API size_t marlin_packed_meta_bytes(int K, int N);
 /* Bytes of the workspace marlin_gemm* needs for any M <= max_M on this K x N layer.
- * The workspace holds a status word, per-column-tile arrival counters and the fp32 partial tiles
- * of the stripe fix-up (the global reduction of Section 3.4 "Striped Partitioning"): a part of fixed size
- * (10.5 MB) and one that grows with N and with max_M up to 128 rows and, above, with the number of
- * (column tile, 128-row slab) pairs up to the number of CTAs (at most 20 MB more).
+ * The workspace holds a status word, arrival counters and slots for the fp32 partial tiles
+ * of the fix-up (the global reduction of Section 3.4 "Striped Partitioning"): at least 10.5 MB, and two slots of
+ * 256 columns x 32, 64 or 128 rows per CTA that a batch of max_M rows can use (at most 42 MB).
  * The caller zeroes it ONCE after allocation (cudaMemset); every call leaves the counters zero.
  * One workspace must not be used by two calls that can run at the same time.  It may serve calls on
  * different layers, formats and batch sizes one after the other (one stream, or ordered by events) if it
@@ -128,18 +127,15 @@ MARLIN_API int marlin_unpack_zeros(const void* z_packed, uint8_t* zeros, int K, 
  *   workspace  device, at least marlin_workspace_bytes(M, K, N) bytes, zeroed once by the caller
  * Accumulation is fp32 (also across stripes) and the result is rounded to fp16 once (nearest even).  The
  * weights reach the tensor cores as exact integers q - 8 (warp-level kernel, up to 16 rows: scales applied to
- * the fp32 sums per group) or as fp16((q - 8) * s) (tcgen05 kernel with in-loop scales, from 17 rows: one more
- * rounding of 2^-11 per weight, as in the paper's kernel).
- * Up to 16 rows the warp-level kernel runs and the same inputs give the same bits on every call.
- * From 17 rows a tcgen05 kernel takes over.  Where N is a multiple of 256 one launch takes all rows: above
+ * the fp32 sums per group; tcgen05 kernel where there is one scale per column or N is not a multiple of 256: scales
+ * applied to fp32 sums too) or as fp16((q - 8) * s) (tcgen05 kernel otherwise: one more rounding of 2^-11 per
+ * weight, as in the paper's kernel).
+ * Up to 16 rows the warp-level kernel runs, from 17 rows (from nine on layers of more than 2^26 weights with one scale
+ * per column) a tcgen05 kernel.  That one takes all rows in one launch: above
  * 128 rows the layer is replicated in the numbering of the work units, once per slab of 128 rows (Section 3.4,
  * last paragraph), and the stripes of the CTAs run over (column tile, slab, k-block), so the weights come from
- * DRAM once and from the L2 after that.  Where N is a multiple of 128 only, 64 rows per launch; any other N goes
- * through the warp-level kernel in slabs of 16 rows.  Groups of 64 or 32 rows run on the tcgen05 kernel at
- * every batch size.  Where the 256-column tcgen05 kernel adds the partial sums of a column tile shared by
- * several CTAs through the L2 (up to 32 rows, above 128 rows, or shapes whose CTAs do not fit as one wave of
- * thread-block clusters) the fp32 additions happen in arrival order, so the last bit of an fp16 result can
- * differ between two calls; everywhere else the order is fixed.
+ * DRAM once and from the L2 after that.  Groups of 64 or 32 rows run on it at every batch size.
+ * Partial sums are added in a fixed order everywhere: the same inputs give the same bits on every call.
  * Errors: argument checks return before anything is queued.  A kernel whose bounded waits expire
  * sets the workspace status word; read it with marlin_read_status. */
 MARLIN_API int marlin_gemm(const void* A, const void* w_packed, const void* s_packed, void* C,
@@ -188,7 +184,7 @@ MARLIN_API int marlin_gemm_w8(const void* A, const void* w_packed, const void* s
                    int group_size, void* workspace, size_t workspace_bytes, marlin_stream stream);
 
 /* The layer with zero points: C = A . W, W[k][n] = (q[k][n] - z[k/G][n]) * s[k/G][n].  Arguments as marlin_gemm, plus
- * z_packed from marlin_pack_zeros.  Up to 16 rows (and in slabs of 16 rows where N is not a multiple of 256) the
+ * z_packed from marlin_pack_zeros.  Up to 16 rows the
  * warp-level kernel runs: the weights enter the MMAs as for the symmetric layer and one more MMA per 16 rows of k,
  * with an all-ones weight operand, gives sum_k a[k][m] per group, so that the group closes with
  * s * (sum_k a (q - 8) + (8 - z) sum_k a).  Above, the tcgen05 kernel, where the zero point replaces the constant 8
