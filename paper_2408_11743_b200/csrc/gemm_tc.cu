@@ -28,8 +28,14 @@ TcPlan plan_tile(int nt, int scale, int rows, int slabs, int kb, int N, int sm_c
   TcPlan best{};
   const long long sms = sm_count < kMaxWorkers ? sm_count : kMaxWorkers;
   const long long ncols = (long long)((N + 128 * nt - 1) / (128 * nt)) * slabs, units = ncols * kb;
-  const double u = per_kb * (nt == 1 ? (rows > 64 ? (scale == tc::kDeferred ? 0.50 : 0.33) : rows > 32 && scale == tc::kDeferred ? 0.40 : 0.30)
+  double u = per_kb * (nt == 1 ? (rows > 64 ? (scale == tc::kDeferred ? 0.50 : 0.33) : rows > 32 && scale == tc::kDeferred ? 0.40 : 0.30)
                                      : (rows > 64 ? 0.66 : rows > 32 ? 0.55 : 0.43));
+  // Several slabs: a 128-column tile fetches the activations of a k-block for half as many MMAs as a 256-column one.  That tells where
+  // the MMAs are short (2:4: 3634 x 10112 x 4864 265 us with 128 columns, 186 with 256; 1024 x 8192 x 8192 83 / 70; but 512 x
+  // 4096 x 11008 32 / 42, whose 256-column tiles divide the SMs badly), and where the activations outgrow the L2's nearer
+  // half (4-bit, 3634 x 10112 x 4864: 350 / 304 us; 2048 x 4096 x 22016: 293 / 309).
+  if (slabs > 1 && per_kb < 1.0) u = nt == 1 ? 0.36 : 0.56;
+  if (slabs > 1 && per_kb >= 1.0 && nt == 1 && (double)slabs * rows * kb * 256.0 > 48e6) u *= 1.2;
   const double fixed = per_kb < 1.0 && nt == 1 ? 0.6 : 0.0;  // (2:4: three copies per k-block instead of two)
   const double exchange = 0.5 + 5.0 * rows / 128 * nt / 2;
   const char* e = getenv("MARLIN_B200_TC_SPLIT");    // tuning knob: 0 forces stripes, 1.. = that many k-ranges per tile
