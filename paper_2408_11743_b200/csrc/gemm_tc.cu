@@ -34,7 +34,7 @@ TcPlan plan_tile(int nt, int scale, int rows, int slabs, int kb, int N, int sm_c
   // the MMAs are short (2:4: 3634 x 10112 x 4864 265 us with 128 columns, 186 with 256; 1024 x 8192 x 8192 83 / 70; but 512 x
   // 4096 x 11008 32 / 42, whose 256-column tiles divide the SMs badly), and where the activations outgrow the L2's nearer
   // half (4-bit, 3634 x 10112 x 4864: 350 / 304 us; 2048 x 4096 x 22016: 293 / 309).
-  if (slabs > 1 && per_kb < 1.0) u = nt == 1 ? 0.36 : 0.56;
+  if (slabs > 1 && per_kb < 1.0) u = nt == 1 ? 0.34 : 0.56;
   if (slabs > 1 && per_kb >= 1.0 && nt == 1 && (double)slabs * rows * kb * 256.0 > 48e6) u *= 1.2;
   const double fixed = per_kb < 1.0 && nt == 1 ? 0.6 : 0.0;  // (2:4: three copies per k-block instead of two)
   const double exchange = 0.5 + 5.0 * rows / 128 * nt / 2;
@@ -66,7 +66,8 @@ TcPlan plan_tile(int nt, int scale, int rows, int slabs, int kb, int N, int sm_c
   if (forced <= 0 || !best.nt) {
     const double n = (double)units / (double)workers;
     const double contributors = (double)workers / (double)ncols + 1.0;
-    take(workers, 0, 0, false, u * n + exchange * (0.5 + 0.7 * (contributors < 2.0 ? 2.0 : contributors)));
+    // (2:4 with several slabs: 218 us in stripes, 186 with whole tiles, 3634 x 10112 x 4864)
+    take(workers, 0, 0, false, u * (slabs > 1 && per_kb < 1.0 ? 1.3 : 1.0) * n + exchange * (0.5 + 0.7 * (contributors < 2.0 ? 2.0 : contributors)));
   }
   // stripes cut at tile boundaries: nothing is shared
   if (forced < 0 && ncols >= workers) take(workers, 0, 0, true, u * (double)((ncols + workers - 1) / workers * kb));
