@@ -188,6 +188,10 @@ template <bool V>
 struct BoolC {
   static constexpr bool value = V;
 };
+template <int V>
+struct IntC {
+  static constexpr int value = V;
+};
 
 // ---- the kernel ---------------------------------------------------------------------------------------------------
 template <int NT, int MPAD, int SCALE, int FMT>
@@ -804,6 +808,47 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
       __syncwarp();
       if (lane == 0) mbar_arrive(&dempty[d]);
     };
+    // A finished tile to C: its fp16 blocks (eight rows x 32 channels in fragment order) into this warp's buffers, several of them
+    // (put_block), then from there to C in runs of 64 bytes (write_blocks; 32 with the fused activation, applied on the way).
+    // These warps get the issue slots that the converters leave: block after block, each a store, a warp barrier, a load and a store
+    // to C that wait for one another, a tile of 128 rows took 4000 to 7000 cycles, and with two tiles the MMAs of the next
+    // segment waited for the accumulators of the second one meanwhile (2:4, 2300 x 1024 x 4096: 21.9 us so, 15.7 this way;
+    // 2048 x 4096 x 22016 226 / 218; 4-bit, 2048 x 1024 x 8192 44.7 / 38.4; 100 x 4096 x 12288 17.0 / 16.2).
+    // The buffers of the converting warps are free here: those use theirs behind the block's barriers only.
+    constexpr int kBufBlocks = imin(RBG, G::OUT_BYTES / G::DRAIN_WARPS / 512);
+    const uint32_t tile_buf = smem_u32(smem) + G::BAR_BYTES + (uint32_t)((warp - G::CONV_WARPS) * kBufBlocks * 512);
+    const uint32_t put_at = tile_buf + (uint32_t)((lane & 7) * 64 + (((lane >> 3) ^ ((lane >> 1) & 3)) * 16));
+    auto put_block = [&](int x, const uint32_t (&r)[4]) { stmatrix_x4_trans(put_at + (uint32_t)(x * 512), r); };
+    auto write_blocks = [&](auto count_c, int b0, int m_lim, size_t row0, uint32_t n0) {
+      constexpr int COUNT = decltype(count_c)::value;
+      __syncwarp();
+      if (!p.swiglu) {
+        const int row = lane >> 2, ch = lane & 3;
+        const uint32_t from = tile_buf + (uint32_t)(row * 64 + ((ch ^ ((row >> 1) & 3)) * 16));
+        uint16_t* c = p.C + (row0 + (size_t)(8 * b0 + row)) * ldc + n0 + ch * 8;
+#pragma unroll
+        for (int x = 0; x < COUNT; x += imin(COUNT, 4)) {
+          uint4 v[imin(COUNT, 4)];
+#pragma unroll
+          for (int y = 0; y < imin(COUNT, 4); ++y) v[y] = lds128(from + (uint32_t)((x + y) * 512));
+#pragma unroll
+          for (int y = 0; y < imin(COUNT, 4); ++y)
+            if ((b0 + x + y) * 8 + row < m_lim) *reinterpret_cast<uint4*>(c + (size_t)(8 * (x + y)) * ldc) = v[y];
+        }
+      } else {
+        // two blocks at a time; of every 16 channels the gate piece and the up piece of a row lie side by side
+        const int row = (lane & 15) >> 1, ch = lane & 1, half = lane >> 4;
+        const uint32_t at = tile_buf + (uint32_t)(half * 512 + row * 64), turn = (uint32_t)((row >> 1) & 3);
+        const uint32_t gate = at + (((uint32_t)(2 * ch) ^ turn) * 16), up = at + (((uint32_t)(2 * ch + 1) ^ turn) * 16);
+        uint16_t* c = p.C + (row0 + (size_t)(8 * (b0 + half) + row)) * ldc + n0 / 2 + ch * 8;
+#pragma unroll
+        for (int x = 0; x < COUNT; x += 2) {
+          const uint4 v = swiglu8(lds128(gate + (uint32_t)(x * 512)), lds128(up + (uint32_t)(x * 512)));
+          if ((b0 + x + half) * 8 + row < m_lim) *reinterpret_cast<uint4*>(c + (size_t)(8 * x) * ldc) = v;
+        }
+      }
+      __syncwarp();  // everybody has read: the buffers may be written again
+    };
     uint32_t it = 0, seg = 0;
     bool waited_for_prior_grid = false;
     for (uint32_t u = u0; u < u1; ++seg) {
@@ -905,12 +950,15 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
                     make_float4(acc[8 * b + 4 * h], acc[8 * b + 4 * h + 1], acc[8 * b + 4 * h + 2], acc[8 * b + 4 * h + 3]);
         } else if (ncol0 < (uint32_t)p.N) {
 #pragma unroll
-          for (int b = 0; b < RBG; ++b)
+          for (int b = 0; b < RBG; b += kBufBlocks)
             if ((b_first + b) * 8 < m_lim) {
-              uint32_t r[4];
-              pack8(acc + 8 * b, r);
-              activate(r);
-              emit(r, buf_s + (uint32_t)(b & 1) * 512, (b_first + b) * 8, m_lim, row0, ncol0);
+#pragma unroll
+              for (int x = 0; x < kBufBlocks; ++x) {
+                uint32_t r[4];
+                pack8(acc + 8 * (b + x), r);
+                put_block(x, r);
+              }
+              write_blocks(IntC<kBufBlocks>{}, b_first + b, m_lim, row0, ncol0);
             }
         }
       } else {
@@ -962,27 +1010,37 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
                         make_float4(f[8 * b + 4 * h], f[8 * b + 4 * h + 1], f[8 * b + 4 * h + 2], f[8 * b + 4 * h + 3]);
             }
           } else {
-            // out of tensor memory as fp16 first: the MMAs of the next segment may start while C is written
-            uint32_t r[RB][4];
+            // All of it out of tensor memory as fp16 first, as much as fits into the buffers and the rest into registers: the
+            // MMAs of the next segment may start while C is written.
+            constexpr int REST = RB - kBufBlocks;
+            uint32_t rest[REST > 0 ? REST : 1][4];
 #pragma unroll
             for (int m = 0; m < MPAD; m += 16) {
               float f[16];
               load_rows(m, f);
-              pack8(f, r[m / 8]);
-              pack8(f + 8, r[m / 8 + 1]);
+#pragma unroll
+              for (int b = 0; b < 2; ++b) {
+                const int x = m / 8 + b;
+                uint32_t r[4];
+                pack8(f + 8 * b, r);
+                if (x < kBufBlocks) {
+                  put_block(x, r);
+                } else {
+#pragma unroll
+                  for (int e = 0; e < 4; ++e) rest[x - kBufBlocks][e] = r[e];
+                }
+              }
             }
             release(t);
             if (n0 < (uint32_t)p.N) {
-              if (p.swiglu) {
+              write_blocks(IntC<kBufBlocks>{}, 0, m_lim, row0, n0);
+              if constexpr (REST > 0) {
+                if (kBufBlocks * 8 < m_lim) {
 #pragma unroll
-                for (int b = 0; b < RB; ++b) {
-                  activate(r[b]);
-                  asm volatile("" : "+r"(r[b][0]), "+r"(r[b][1])::"memory");  // one block after the other, to spare registers
+                  for (int x = 0; x < REST; ++x) put_block(x, rest[x]);
+                  write_blocks(IntC<REST>{}, kBufBlocks, m_lim, row0, n0);
                 }
               }
-#pragma unroll
-              for (int b = 0; b < RB; ++b)
-                if (b * 8 < m_lim) emit(r[b], buf_s + (uint32_t)(b & 1) * 512, b * 8, m_lim, row0, n0);
             }
           }
         }

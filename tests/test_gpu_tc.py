@@ -7,7 +7,7 @@ import numpy as np
 import pytest
 
 from paper_2408_11743_b200 import inputs
-from gpu_util import DenseLayer, SparseLayer
+from gpu_util import DenseLayer, SparseLayer, to_dev, to_host
 
 pytestmark = pytest.mark.gpu
 
@@ -85,3 +85,56 @@ def test_large_layers_with_one_scale_per_column_change_kernels_at_nine_rows(marl
     C = layer(case.A)
     bad, worst, rms = oracle_lib.check_tolerance(C, oracle_lib.gemm(case.A, case.q_kpacked, case.S, case.G))
     assert bad == 0, (bad, worst, rms)
+
+
+# Finished tiles go to C through buffers of several blocks of eight rows: rows at the edges of a block, of a buffer (64) and of a
+# slab, one tile per CTA and several, whole and narrow last tiles.  C lies in a larger buffer whose surroundings must survive.
+@pytest.mark.parametrize("M,K,N,G,split", [
+    (17, 256, 256, 128, "1"), (31, 256, 320, 128, "1"), (33, 256, 512, -1, "1"), (63, 384, 320, -1, "1"), (65, 256, 512, 128, "1"),
+    (72, 256, 576, 128, "1"), (121, 512, 256, 64, "1"), (127, 256, 1344, 256, "1"), (137, 256, 768, 128, "1"),
+    (250, 128, 320, 128, "1"), (300, 256, 12800, 128, None), (130, 128, 22016, -1, None), (200, 256, 10304, 128, None)])
+@pytest.mark.parametrize("tile", ["128", "256"])
+def test_every_row_of_c_and_nothing_else_is_written(marlin, oracle_lib, monkeypatch, tile, M, K, N, G, split):
+    import torch
+    monkeypatch.setenv("MARLIN_B200_TC_TILE", tile)
+    if split:
+        monkeypatch.setenv("MARLIN_B200_TC_SPLIT", split)
+    rng = np.random.default_rng(M + N)
+    Gn = K if G == -1 else G
+    Q = rng.integers(0, 16, size=(K, N), dtype=np.uint8)
+    A = rng.integers(-3, 4, size=(M, K)).astype(np.float16)
+    S = np.ldexp(1.0, rng.integers(-4, 1, size=(K // Gn, N))).astype(np.float16)
+    q = inputs.kpack(Q)
+    layer = DenseLayer(marlin, q, S, G, max_M=M)
+    guard = 64 * N
+    big = torch.full((2 * guard + M * N,), float("nan"), dtype=torch.float16, device="cuda")
+    out = big[guard:guard + M * N].view(M, N)
+    marlin.gemm(to_dev(A), layer.w, layer.s, K, N, G, layer.ws, out=out)
+    torch.cuda.synchronize()
+    assert marlin.read_status(layer.ws) == 0
+    want = (A.astype(np.float64) @ ((Q.astype(np.float64) - 8) * np.repeat(S.astype(np.float64), Gn, axis=0))).astype(np.float16)
+    assert np.array_equal(to_host(out), want)  # integers times powers of two: every partial sum is exact
+    assert bool(big[:guard].isnan().all()) and bool(big[guard + M * N:].isnan().all())
+
+
+# the fused activation on the way out: H against silu(g) * u of the g and u that the same layer gives without it.  Bound: one
+# rounding to fp16 (2^-11) and the fp32 exponential and division (below 2^-18 for |g| < 88): 2^-10.9 of |H|, and half of the smallest fp16.
+@pytest.mark.parametrize("M,I,G", [(17, 128, 128), (40, 160, 128), (72, 672, 128), (121, 128, 64), (129, 256, -1), (250, 160, -1),
+                                   (300, 6400, 128)])
+def test_fused_activation_on_the_way_out(marlin, M, I, G):
+    import torch
+    K, N = 256, 2 * I
+    case = inputs.make_dense(M, K, N, G, seed=M + I)
+    layer = DenseLayer(marlin, case.q_kpacked, case.S, G, max_M=M)
+    A = to_dev(case.A)
+    C = to_host(marlin.gemm(A, layer.w, layer.s, K, N, G, layer.ws)).astype(np.float64).reshape(M, I // 8, 2, 8)
+    guard = 64 * I
+    big = torch.full((2 * guard + M * I,), float("nan"), dtype=torch.float16, device="cuda")
+    H = big[guard:guard + M * I].view(M, I)
+    marlin.gemm_swiglu(A, layer.w, layer.s, K, N, G, layer.ws, out=H)
+    torch.cuda.synchronize()
+    g, u = C[:, :, 0].reshape(M, I), C[:, :, 1].reshape(M, I)
+    want = g / (1 + np.exp(-g)) * u
+    err = np.abs(to_host(H).astype(np.float64) - want)
+    assert np.all(err <= 2.0 ** -10.9 * np.abs(want) + 2.0 ** -25 + 1e-9)
+    assert bool(big[:guard].isnan().all()) and bool(big[guard + M * I:].isnan().all())
