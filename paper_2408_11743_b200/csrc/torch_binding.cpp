@@ -11,6 +11,7 @@
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/autograd/python_variable.h>
 
+#include <climits>
 #include <cstdint>
 
 namespace {
@@ -32,6 +33,18 @@ MlpFn g_mlp;
 SizeFn g_weight_bytes, g_scale_bytes;
 SizeFn2 g_meta_bytes, g_weight_bytes_w8;
 PyObject* g_raise;  // raise(status, what)
+
+// an argument as the int that the library takes; false with a Python error set (a size beyond it is no other size)
+bool integer(PyObject* o, const char* name, int* out) {
+  const long v = PyLong_AsLong(o);
+  if (v == -1 && PyErr_Occurred()) return false;
+  if (v < INT_MIN || v > INT_MAX) {
+    PyErr_Format(PyExc_ValueError, "%s is out of range", name);
+    return false;
+  }
+  *out = (int)v;
+  return true;
+}
 
 // nullptr with a Python error set, or the tensor
 const at::Tensor* tensor(PyObject* o, const char* name) {
@@ -206,9 +219,9 @@ PyObject* make_layer_call(PyObject*, PyObject* args) {
 PyObject* gemm(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
   TRY
   if (!count_is(nargs, 11)) return nullptr;
-  const int kind = (int)PyLong_AsLong(a[0]), K = (int)PyLong_AsLong(a[5]), N = (int)PyLong_AsLong(a[6]),
-            G = (int)PyLong_AsLong(a[7]);
-  if (PyErr_Occurred()) return nullptr;
+  int kind, K, N, G;
+  if (!integer(a[0], "kind", &kind) || !integer(a[5], "K", &K) || !integer(a[6], "N", &N) || !integer(a[7], "group_size", &G))
+    return nullptr;
   const at::Tensor* A = activations(a[1], K);
   if (!A) return nullptr;
   const at::Tensor* w = device_tensor(a[2], at::kByte, "w_packed");
@@ -241,9 +254,9 @@ PyObject* gemm(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
 PyObject* mlp(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
   TRY
   if (!count_is(nargs, 13)) return nullptr;
-  const int K = (int)PyLong_AsLong(a[5]), I = (int)PyLong_AsLong(a[6]), N = (int)PyLong_AsLong(a[7]),
-            G = (int)PyLong_AsLong(a[8]);
-  if (PyErr_Occurred()) return nullptr;
+  int K, I, N, G;
+  if (!integer(a[5], "K", &K) || !integer(a[6], "I", &I) || !integer(a[7], "N", &N) || !integer(a[8], "group_size", &G))
+    return nullptr;
   const at::Tensor* A = activations(a[0], K);
   if (!A) return nullptr;
   const at::Tensor* ws = device_tensor(a[9], at::kByte, "workspace");

@@ -413,6 +413,27 @@ def test_native_binding_refuses_what_the_kernels_cannot_take(marlin, bad, error)
             marlin.Layer(w, layer.s, 256, 192, 128, layer.ws)(A, out=out)
 
 
+# sizes that do not fit into the C ABI's int are refused, not cut to their low 32 bits (which would be this layer)
+@pytest.mark.parametrize("dK,dN,dG", [(1 << 32, 0, 0), (0, 1 << 32, 0), (0, 0, 1 << 32), (-(1 << 32), 0, 0), (1 << 64, 0, 0)])
+def test_sizes_beyond_32_bits_are_refused(marlin, dK, dN, dG):
+    import torch
+    case = inputs.make_dense(4, 256, 192, 128, seed=3)
+    layer = DenseLayer(marlin, case.q_kpacked, case.S, 128, max_M=4)
+    A = to_dev(case.A)
+    out = torch.empty((4, 192), dtype=torch.float16, device="cuda")
+    refused = (ValueError, OverflowError)
+    with pytest.raises(refused):
+        marlin.gemm(A, layer.w, layer.s, 256 + dK, 192 + dN, 128 + dG, layer.ws, out=out)
+    up, down = inputs.make_dense(4, 256, 256, 128, seed=4), inputs.make_dense(4, 128, 192, 128, seed=5)
+    wu, wd = (DenseLayer(marlin, c.q_kpacked, c.S, 128, max_M=4) for c in (up, down))
+    mlp = (wu.w, wu.s, wd.w, wd.s)
+    assert marlin.mlp_swiglu(A, *mlp, 256, 128, 192, 128, wu.ws, out=out) is out
+    with pytest.raises(refused):
+        marlin.mlp_swiglu(A, *mlp, 256 + dK, 128, 192 + dN, 128 + dG, wu.ws, out=out)
+    with pytest.raises(refused):
+        marlin.Layer(layer.w, layer.s, 256 + dK, 192 + dN, 128 + dG, layer.ws)(A, out=out)
+
+
 # teams of CTAs with several column tiles each: one and two CTAs, 64- and 128-column tiles, teams of unequal size, both block
 # counts, exchange through clusters and through the workspace
 @pytest.mark.parametrize("M,K,N,mode", [
