@@ -86,7 +86,6 @@ def lib():
     return L
 
 
-_NATIVE_PATH = os.path.join(_HERE, "_torch_binding.so")
 _native = None
 
 
@@ -96,10 +95,11 @@ def native():
     global _native
     if _native is not None:
         return _native
-    if not os.path.exists(_NATIVE_PATH):
-        raise RuntimeError(f"{_NATIVE_PATH} is missing: build it with `python -m paper_2408_11743_b200.build`")
-    _torch()  # the module uses the libraries that torch has loaded
-    spec = importlib.util.spec_from_file_location("_torch_binding", _NATIVE_PATH)
+    from .build import native_path
+    path = native_path()  # (imports torch, whose libraries the module uses)
+    if not os.path.exists(path):
+        raise RuntimeError(f"{path} is missing: build it with `python -m paper_2408_11743_b200.build`")
+    spec = importlib.util.spec_from_file_location("_torch_binding", path)
     mod = importlib.util.module_from_spec(spec)
     spec.loader.exec_module(mod)
     L = lib()

@@ -34,27 +34,41 @@ def _nvcc() -> str:
 
 
 # the per-call part of the Python binding: host code against torch's C++ API
-NATIVE = os.path.join(_HERE, "_torch_binding.so")
 NATIVE_SOURCE = os.path.join(CSRC, "torch_binding.cpp")
 
 
-def build_native(force: bool = False, verbose: bool = False) -> str:
+def native_path() -> str:
+    """Where the extension module for this Python and this torch lies.  It is compiled against the C++ headers of the one
+    and the object layouts of the other, so both are part of its name: after an upgrade the old file is not found (and
+    not loaded) instead of misreading tensors."""
+    import re
     import sysconfig
+    import torch
+    tag = f"{sysconfig.get_config_var('SOABI')}-torch-{torch.__version__}-abi{int(torch._C._GLIBCXX_USE_CXX11_ABI)}"
+    return os.path.join(_HERE, "_torch_binding." + re.sub(r"[^\w.+-]", "_", tag) + ".so")
+
+
+def build_native(force: bool = False, verbose: bool = False) -> str:
+    import glob
+    import sysconfig
+    native = native_path()
     deps = [NATIVE_SOURCE, os.path.abspath(__file__)]
-    if not force and os.path.exists(NATIVE) and all(os.path.getmtime(d) <= os.path.getmtime(NATIVE) for d in deps):
-        return NATIVE
+    if not force and os.path.exists(native) and all(os.path.getmtime(d) <= os.path.getmtime(native) for d in deps):
+        return native
     import torch
     t = os.path.dirname(torch.__file__)
     cuda = os.path.dirname(os.path.dirname(_nvcc())) if os.path.isabs(_nvcc()) else "/usr/local/cuda"
+    for old in glob.glob(os.path.join(_HERE, "_torch_binding*.so")):
+        os.remove(old)
     cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-fvisibility=hidden", "-shared",
            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
            "-isystem", os.path.join(t, "include"), "-isystem", os.path.join(t, "include", "torch", "csrc", "api", "include"),
-           "-isystem", sysconfig.get_paths()["include"], "-isystem", os.path.join(cuda, "include"), NATIVE_SOURCE, "-o", NATIVE,
+           "-isystem", sysconfig.get_paths()["include"], "-isystem", os.path.join(cuda, "include"), NATIVE_SOURCE, "-o", native,
            "-L", os.path.join(t, "lib"), "-ltorch_python", "-ltorch_cuda", "-ltorch_cpu", "-lc10_cuda", "-lc10"]
     if verbose:
         print(" ".join(cmd), flush=True)
     subprocess.run(cmd, check=True)
-    return NATIVE
+    return native
 
 
 def needs_build() -> bool:

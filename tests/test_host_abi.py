@@ -37,6 +37,26 @@ def test_missing_library_fails_loudly(monkeypatch, marlin):
         binding.lib()
 
 
+def test_extension_module_of_another_torch_or_python_is_not_loaded(monkeypatch, marlin):
+    # it is compiled against torch's headers and Python's object layouts: with another version of either it must count as missing
+    import sysconfig
+    import torch
+    from paper_2408_11743_b200 import binding, build
+    path = build.native_path()
+    assert os.path.exists(path)
+    monkeypatch.setattr(binding, "_native", None)
+    with monkeypatch.context() as m:
+        m.setattr(torch, "__version__", "1.0.0")
+        assert build.native_path() != path
+        with pytest.raises(RuntimeError, match="missing"):
+            binding.native()
+    real = sysconfig.get_config_var
+    with monkeypatch.context() as m:
+        m.setattr(sysconfig, "get_config_var", lambda name: "cpython-30" if name == "SOABI" else real(name))
+        with pytest.raises(RuntimeError, match="missing"):
+            binding.native()
+
+
 def test_size_queries(marlin):
     L = marlin.lib()
     assert L.marlin_packed_weight_bytes(4096, 4096, 0) == 4096 * 4096 // 2
