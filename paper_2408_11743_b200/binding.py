@@ -390,21 +390,8 @@ def unpack_sparse24(w_packed, meta_packed, s_packed, K: int, N: int, group_size:
 
 def gemm_sparse24(A, w_packed, meta_packed, s_packed, K: int, N: int, group_size: int, workspace, out=None,
                   stream=None):
-    torch = _torch()
-    A = _dev(A, torch.float16, "A")
-    if A.dim() != 2 or A.shape[1] != K:
-        raise ValueError("A must be [M, K]")
-    M = A.shape[0]
-    w = _dev(w_packed, torch.uint8, "w_packed")
-    m = _dev(meta_packed, torch.uint8, "meta_packed")
-    s = _dev(s_packed, torch.uint8, "s_packed")
-    ws = _dev(workspace, torch.uint8, "workspace")
-    if out is None:
-        out = torch.empty((M, N), dtype=torch.float16, device=A.device)
-    _check(lib().marlin_gemm_sparse24(A.data_ptr(), w.data_ptr(), m.data_ptr(), s.data_ptr(), out.data_ptr(), M, K,
-                                      N, group_size, ws.data_ptr(), ws.numel(), _stream_ptr(stream)),
-           "marlin_gemm_sparse24")
-    return out
+    """marlin_gemm_sparse24: C = A . W for a 2:4 layer (see pack_sparse24)."""
+    return native().gemm(_SPARSE, A, w_packed, s_packed, meta_packed, K, N, group_size, workspace, out, stream)
 
 
 class Layer:

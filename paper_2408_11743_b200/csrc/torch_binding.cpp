@@ -215,7 +215,7 @@ PyObject* make_layer_call(PyObject*, PyObject* args) {
 }
 
 // ---- the module-level functions ---------------------------------------------------------------------------------
-// gemm(kind, A, w_packed, s_packed, extra or None, K, N, G, workspace, out or None, stream or None)
+// gemm(kind, A, w_packed, s_packed, metadata, zero points or None, K, N, G, workspace, out or None, stream or None)
 PyObject* gemm(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
   TRY
   if (!count_is(nargs, 11)) return nullptr;
@@ -229,7 +229,8 @@ PyObject* gemm(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
   const at::Tensor* s = device_tensor(a[3], at::kByte, "s_packed");
   if (!s) return nullptr;
   const at::Tensor* x = nullptr;
-  if (a[4] != Py_None && !(x = device_tensor(a[4], at::kByte, kind == kSparse ? "meta_packed" : "z_packed"))) return nullptr;
+  if ((kind == kSparse || kind == kZero) && !(x = device_tensor(a[4], at::kByte, kind == kSparse ? "meta_packed" : "z_packed")))
+    return nullptr;
   const at::Tensor* ws = device_tensor(a[8], at::kByte, "workspace");
   if (!ws) return nullptr;
   const size_t wb = kind == kW8 ? g_weight_bytes_w8(K, N) : g_weight_bytes(K, N, kind == kSparse ? 1 : 0);

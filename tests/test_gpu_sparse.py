@@ -159,3 +159,28 @@ def test_config5_full_size_on_sampled_outputs(marlin, oracle_lib):
     ref = oracle_lib.gemm_samples(case.A, inputs.kpack(Q), case.S, G, ms, ns)
     bad, worst, _ = oracle_lib.check_tolerance(np.ascontiguousarray(C[ms, ns]), ref)
     assert bad == 0, worst
+
+
+# buffers that do not fit the layer, and outputs that are not C, are refused before anything is launched
+@pytest.mark.parametrize("bad,error", [("w", ValueError), ("meta", ValueError), ("s", ValueError), ("no_meta", TypeError),
+                                       ("meta_cpu", TypeError), ("out_rows", ValueError), ("out_dtype", TypeError),
+                                       ("out_cpu", TypeError), ("out_strided", ValueError)])
+def test_buffers_and_outputs_that_do_not_fit_are_refused(marlin, bad, error):
+    import torch
+    M, K, N, G = 4, 512, 256, 128
+    case = inputs.make_sparse24(M, K, N, G, seed=5)
+    L = SparseLayer(marlin, case, M)
+    A, w, meta, s = to_dev(case.A), L.w, L.meta, L.s
+    out = torch.empty((M, N), dtype=torch.float16, device="cuda")
+    assert marlin.gemm_sparse24(A, w, meta, s, K, N, G, L.ws, out=out) is out
+    if bad == "w": w = w[:-16]
+    if bad == "meta": meta = meta[:-16]
+    if bad == "s": s = s[:-16]
+    if bad == "no_meta": meta = None
+    if bad == "meta_cpu": meta = meta.cpu()
+    if bad == "out_rows": out = out[:-1]
+    if bad == "out_dtype": out = out.float()
+    if bad == "out_cpu": out = out.cpu()
+    if bad == "out_strided": out = torch.empty((N, M), dtype=torch.float16, device="cuda").t()
+    with pytest.raises(error):
+        marlin.gemm_sparse24(A, w, meta, s, K, N, G, L.ws, out=out)
