@@ -6,7 +6,7 @@
 namespace marlin_b200 {
 
 // how the weights reach the MMAs, as far as the cost of a k-block goes
-enum TcFormat { kTcDense4 = 0, kTcSparse4 = 1, kTcDense8 = 2, kTcDeferred4 = 3 };
+enum TcFormat { kTcDense4 = 0, kTcSparse4 = 1, kTcDense8 = 2, kTcDeferred4 = 3, kTcZero4 = 4 };
 
 // rows of a slab: the MMA's N
 inline int tc_mpad(int m) { return m <= 32 ? 32 : (m <= 64 ? 64 : 128); }
@@ -38,18 +38,20 @@ struct TcPlan {
 // fastest one and more than 5 % on 36 pairs.  The constants before it (from about a dozen shapes, nothing per tile, the 8-bit ones
 // scaled from 4-bit, 1.8 us for a small grid) missed by 2.6 % and, by more than 5 %, on 212 of 1198: 28672 x 8192 at 48 rows
 // 46 us, 35 now (256 columns and four k-ranges instead of 128 and two); 8-bit at 256 rows 145 / 113; 2:4, 1024 x 14336 at 128 rows
-// 11.5 / 8.0; 4096 x 22016 at 64 rows 18.5 / 14.4.
+// 11.5 / 8.0; 4096 x 22016 at 64 rows 18.5 / 14.4.  Zero points, whose conversion is longer, have k-blocks of their own: with those
+// of 4-bit the pick is 1.6 % above the fastest on 76 pairs above 128 rows, 0.7 % so (200 x 5120 x 13824 42.3 us, 38.8 now).
 inline TcPlan plan_tc_tile(int nt, int format, int rows, int slabs, int kb, int N, int sm_count, int max_workers) {
   TcPlan best{};
   const long long sms = sm_count < max_workers ? sm_count : max_workers;
   const long long ncols = (long long)((N + 128 * nt - 1) / (128 * nt)) * slabs, units = ncols * kb;
   const int mpad = tc_mpad(rows), mi = mpad == 32 ? 0 : mpad == 64 ? 1 : 2;
   // [format][tiles][32, 64, 128 rows]
-  static const double k_block[4][2][3] = {{{0.252, 0.291, 0.348}, {0.363, 0.431, 0.639}},
+  static const double k_block[5][2][3] = {{{0.252, 0.291, 0.348}, {0.363, 0.431, 0.639}},
                                           {{0.230, 0.296, 0.254}, {0.223, 0.332, 0.373}},
                                           {{0.214, 0.280, 0.352}, {0.354, 0.487, 0.639}},
-                                          {{0.349, 0.504, 0.714}, {0.349, 0.504, 0.714}}};
-  static const double load[4] = {0.152, 0.069, 0.415, 0.0};
+                                          {{0.349, 0.504, 0.714}, {0.349, 0.504, 0.714}},
+                                          {{0.288, 0.341, 0.370}, {0.456, 0.553, 0.826}}};
+  static const double load[5] = {0.152, 0.069, 0.415, 0.0, 0.087};
   static const double read_out[2][3] = {{0.89, 0.53, 1.80}, {1.30, 1.36, 3.35}};
   const double start = 2.09;
   const double tile = read_out[nt - 1][mi] * (rows < mpad / 4 ? 0.25 : (double)rows / mpad);

@@ -8,7 +8,7 @@ import subprocess
 import pytest
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
-DENSE4, SPARSE4, DENSE8, DEFERRED4 = range(4)
+DENSE4, SPARSE4, DENSE8, DEFERRED4, ZERO4 = range(5)
 RESIDENT = [0, 148, 74, 45, 33, 26, 22, 15, 15]  # clusters of that size that a B200 holds at once
 
 SHIM = """
@@ -36,7 +36,7 @@ def plan(tmp_path_factory):
     return ask
 
 
-@pytest.mark.parametrize("fmt", [DENSE4, SPARSE4, DENSE8, DEFERRED4])
+@pytest.mark.parametrize("fmt", [DENSE4, SPARSE4, DENSE8, DEFERRED4, ZERO4])
 @pytest.mark.parametrize("env", [{}, {"MARLIN_B200_TC_SPLIT": "0"}, {"MARLIN_B200_TC_SPLIT": "3"}, {"MARLIN_B200_TC_CLUSTER": "0"},
                                  {"MARLIN_B200_TC_TILE": "256"}])
 def test_every_plan_can_run(plan, monkeypatch, fmt, env):
@@ -82,6 +82,8 @@ def test_every_plan_can_run(plan, monkeypatch, fmt, env):
     (SPARSE4, 384, 1024, 4096, {(1, 1)}),                  # 7.8 / 6.4
     (SPARSE4, 128, 4096, 4096, {(1, 4), (1, 3)}),          # 10.1 / 9.1
     (DEFERRED4, 160, 1024, 14400, {(1, "whole")}),         # 17.7 / 15.8
+    (ZERO4, 200, 5120, 13824, {(1, "whole")}),             # 42.3 / 38.8 with the k-blocks of DENSE4
+    (ZERO4, 777, 11008, 4096, {(1, "whole"), (1, "even")}),  # 86.8 / 80.7
 ])
 def test_picks_among_the_fastest_of_the_timed_candidates(plan, fmt, M, K, N, good):
     p = plan(fmt, M, K, N)
