@@ -39,7 +39,8 @@ struct TcPlan {
 // scaled from 4-bit, 1.8 us for a small grid) missed by 2.6 % and, by more than 5 %, on 212 of 1198: 28672 x 8192 at 48 rows
 // 46 us, 35 now (256 columns and four k-ranges instead of 128 and two); 8-bit at 256 rows 145 / 113; 2:4, 1024 x 14336 at 128 rows
 // 11.5 / 8.0; 4096 x 22016 at 64 rows 18.5 / 14.4.  Zero points, whose conversion is longer, have k-blocks of their own: with those
-// of 4-bit the pick is 1.6 % above the fastest on 76 pairs above 128 rows, 0.7 % so (200 x 5120 x 13824 42.3 us, 38.8 now).
+// of 4-bit the pick is 1.6 % above the fastest on 76 pairs above 128 rows, 0.7 % so (200 x 5120 x 13824 42.3 us, 38.8 now).  Up to 32 rows the constants of 2:4 and zero points and the read-out come from
+// another 200 pairs (2:4, 4096 x 22016 at one row 14.7 us with one k-range per tile, 12.5 in even stripes).
 inline TcPlan plan_tc_tile(int nt, int format, int rows, int slabs, int kb, int N, int sm_count, int max_workers) {
   TcPlan best{};
   const long long sms = sm_count < max_workers ? sm_count : max_workers;
@@ -47,12 +48,12 @@ inline TcPlan plan_tc_tile(int nt, int format, int rows, int slabs, int kb, int 
   const int mpad = tc_mpad(rows), mi = mpad == 32 ? 0 : mpad == 64 ? 1 : 2;
   // [format][tiles][32, 64, 128 rows]
   static const double k_block[5][2][3] = {{{0.252, 0.291, 0.348}, {0.363, 0.431, 0.639}},
-                                          {{0.230, 0.296, 0.254}, {0.223, 0.332, 0.373}},
+                                          {{0.254, 0.296, 0.254}, {0.250, 0.332, 0.373}},
                                           {{0.214, 0.280, 0.352}, {0.354, 0.487, 0.639}},
                                           {{0.349, 0.504, 0.714}, {0.349, 0.504, 0.714}},
-                                          {{0.288, 0.341, 0.370}, {0.456, 0.553, 0.826}}};
+                                          {{0.288, 0.341, 0.370}, {0.454, 0.553, 0.826}}};
   static const double load[5] = {0.152, 0.069, 0.415, 0.0, 0.087};
-  static const double read_out[2][3] = {{0.89, 0.53, 1.80}, {1.30, 1.36, 3.35}};
+  static const double read_out[2][3] = {{1.00, 0.53, 1.80}, {1.70, 1.36, 3.35}};
   const double start = 2.09;
   const double tile = read_out[nt - 1][mi] * (rows < mpad / 4 ? 0.25 : (double)rows / mpad);
   const double exchange = 1.04 + 3.70 * rows / 128 * nt;
@@ -61,7 +62,7 @@ inline TcPlan plan_tc_tile(int nt, int format, int rows, int slabs, int kb, int 
   const char* c = getenv("MARLIN_B200_TC_CLUSTER");  // tuning knob: largest cluster (0: none)
   const int forced = e ? atoi(e) : -1, max_cluster = c ? atoi(c) : 8;
   auto take = [&](long long workers, int split, int cluster, bool whole, double cost) {
-    cost += start - (2 * workers <= sms ? 0.45 : 0.0);
+    cost += start - (2 * workers <= sms ? (mi == 0 ? 0.63 : 0.45) : 0.0);
     if (best.nt && cost >= best.cost) return;
     best = TcPlan{nt, ncols, workers, split, cluster, whole, cost};
   };

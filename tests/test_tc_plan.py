@@ -83,6 +83,9 @@ def test_every_plan_can_run(plan, monkeypatch, fmt, env):
     (SPARSE4, 128, 4096, 4096, {(1, 4), (1, 3)}),          # 10.1 / 9.1
     (DEFERRED4, 160, 1024, 14400, {(1, "whole")}),         # 17.7 / 15.8
     (ZERO4, 200, 5120, 13824, {(1, "whole")}),             # 42.3 / 38.8 with the k-blocks of DENSE4
+    (SPARSE4, 1, 4096, 22016, {(2, "even")}),              # 14.7 / 12.5 with the k-blocks of more rows
+    (SPARSE4, 1, 2048, 8192, {(2, 2)}),                    # 6.2 / 5.6
+    (ZERO4, 22, 4096, 22016, {(2, "even")}),               # 19.5 / 18.1
     (ZERO4, 777, 11008, 4096, {(1, "whole"), (1, "even")}),  # 86.8 / 80.7
 ])
 def test_picks_among_the_fastest_of_the_timed_candidates(plan, fmt, M, K, N, good):
