@@ -174,3 +174,19 @@ def test_one_workspace_serves_layers_of_different_kinds_in_turn(marlin, oracle_l
         assert bad == 0, (i, which, bad, worst)
     host = to_host(ws)
     assert np.all(host[256:8192] == 0)  # arrival counters
+
+
+# nothing reads a slot of the workspace before the same call has written it: NaN in all of them changes no bit
+@pytest.mark.parametrize("mode", range(len(MODES)))
+@pytest.mark.parametrize("M,K,N,G", [(8, 4096, 512, 128), (16, 11008, 1088, 128), (40, 4096, 1024, 128), (24, 16384, 256, -1),
+                                     (64, 2048, 1344, 128), (128, 8192, 576, -1), (300, 2048, 768, 64), (200, 4096, 320, 128)])
+def test_slots_are_written_before_they_are_read(marlin, monkeypatch, mode, M, K, N, G):
+    import torch
+    for k, v in {**MODES[mode], **{k.replace("TC_", ""): v for k, v in MODES[mode].items()}}.items():
+        monkeypatch.setenv(k, v)
+    case = inputs.make_dense(M, K, N, G, seed=M + K + N)
+    layer = DenseLayer(marlin, case.q_kpacked, case.S, G, max_M=M)
+    want = layer(case.A)
+    layer.ws[8192:].view(torch.float32).fill_(float("nan"))
+    assert np.array_equal(layer(case.A).view(np.uint16), want.view(np.uint16))
+    assert np.all(np.isfinite(want.astype(np.float32)))
