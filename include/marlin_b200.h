@@ -257,8 +257,8 @@ MARLIN_API int marlin_read_status(const void* workspace, marlin_stream stream);
  * worker (no stripe crosses a tile boundary); otherwise the units are cut into `workers` even stripes,
  * the paper's form.  Fills n_tile (columns per tile: 64, 128 or 256), workers (<= sm_count) and
  * bounds[0..workers] (host pointers; `cap` entries available in bounds).
- * A launch starts from the same two forms, but may leave some SMs to the next launch or give pairs of
- * workers several column tiles where its cost model finds that faster.
+ * This is the base form.  A launch may take another: fewer CTAs, which leave SMs to the next launch, or pairs of
+ * workers with several column tiles, where its cost model finds that faster.
  * Returns MARLIN_ERR_SHAPE if cap is too small or the shape is invalid. */
 MARLIN_API int marlin_plan_stripes(int M, int K, int N, int sm_count, int* n_tile, int* workers,
                         int64_t* bounds, int cap);

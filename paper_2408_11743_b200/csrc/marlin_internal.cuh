@@ -6,6 +6,7 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include "dense_plan.h"
 #include "marlin_b200.h"
 
 namespace marlin_b200 {
@@ -130,13 +131,6 @@ __device__ inline uint32_t stripe_owner32(uint32_t x, uint32_t U, uint32_t P) { 
 __device__ inline uint32_t split_begin32(uint32_t w, uint32_t KB, uint32_t S) {
   const uint32_t t = w / S, r = w - t * S;
   return t * KB + (r * KB) / S;
-}
-
-// Teams of S workers, C of them (warp-level kernel): the first ncols % C teams own ncols / C + 1 column tiles, the others
-// ncols / C, one team after the other; the workers of a team have even stripes over its k-blocks.  With C = ncols this is the
-// tile-aligned variant above.
-__host__ __device__ inline uint32_t team_first_tile(uint32_t t, uint32_t tiles, uint32_t extra) {
-  return t * tiles + (t < extra ? t : extra);
 }
 
 }  // namespace marlin_b200
