@@ -67,9 +67,10 @@ MARLIN_API size_t marlin_packed_scale_bytes(int K, int N, int group_size);
 MARLIN_API size_t marlin_packed_meta_bytes(int K, int N);
 /* Bytes of the workspace marlin_gemm* needs for any M <= max_M on this K x N layer.
  * The workspace holds a status word, arrival counters and slots for the fp32 partial tiles
- * of the fix-up (the global reduction of Section 3.4 "Striped Partitioning"): at least 10.5 MB, and two slots of
+ * of the fix-up (the global reduction of Section 3.4 "Striped Partitioning"): at least 5.2 MB, and two slots of
  * 256 columns x 32, 64 or 128 rows per CTA that a batch of max_M rows can use (at most 42 MB).
- * The caller zeroes it ONCE after allocation (cudaMemset); every call leaves the counters zero.
+ * The caller zeroes it ONCE after allocation (cudaMemset); every call leaves the counters zero and writes the slots
+ * before it reads them (what they hold between calls is not specified).
  * One workspace must not be used by two calls that can run at the same time.  It may serve calls on
  * different layers, formats and batch sizes one after the other (one stream, or ordered by events) if it
  * has the largest of their sizes: the parts lie at the same offsets for every call. */

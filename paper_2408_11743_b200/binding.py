@@ -247,7 +247,7 @@ def unpack_zeros(z_packed, K: int, N: int, group_size: int, stream=None):
 
 
 def gemm_zp(A, w_packed, s_packed, z_packed, K: int, N: int, group_size: int, workspace, out=None, stream=None):
-    """marlin_gemm_zp: C = A . ((q - z) * s) with per-group zero points; N % 256 == 0."""
+    """marlin_gemm_zp: C = A . ((q - z) * s) with per-group zero points."""
     return native().gemm(_ZERO, A, w_packed, s_packed, z_packed, K, N, group_size, workspace, out, stream)
 
 

@@ -108,6 +108,17 @@ def spill_report():
     return out
 
 
+TC_LAUNCH_REGS = 96  # kLaunchRegs of csrc/gemm_tc.cuh
+
+
+def check_registers(report):
+    """The warps of the tcgen05 kernels share out the registers that a block is launched with, so these kernels launch with
+    exactly that many or not at all: a compiler that takes another number shows here, not in every call."""
+    off = {k: v[0] for k, v in report.items() if "gemm_tc_kernel" in k and v[0] != TC_LAUNCH_REGS}
+    if off:
+        raise RuntimeError(f"tcgen05 kernels compiled to other than {TC_LAUNCH_REGS} registers a thread: {off}")
+
+
 def build(force: bool = False, verbose: bool = False, extra_flags=(), out: str = LIB) -> str:
     """Compiles every .cu of the library and links `out`.  `extra_flags` (for example -DMARLIN_TIMING)
     and a different `out` give an instrumented variant beside the product library."""
@@ -141,6 +152,7 @@ def build(force: bool = False, verbose: bool = False, extra_flags=(), out: str =
     if out == LIB:
         with open(PTXAS_LOG, "w") as f:
             f.write("".join(logs))
+        check_registers(spill_report())
     link = [_nvcc(), "-shared", "-o", out, *objs, "-cudart", "static",
             "-gencode", "arch=compute_100a,code=sm_100a"]
     subprocess.run(link, check=True)

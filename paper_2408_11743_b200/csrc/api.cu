@@ -106,7 +106,8 @@ size_t marlin_packed_meta_bytes(int K, int N) {
 }
 
 // Workspace map: [status word, counters: 8192 bytes][partial-tile slots].  The counters are zero at rest and every kernel
-// leaves them that way; the slots are written before they are read in every call and keep what the last call left.
+// leaves them that way; the slots are written before they are read in every call, and what they hold in between means
+// nothing (the tcgen05 kernel clears most of what it has read, the others leave it).
 // So one buffer may serve calls on different layers, batch sizes and formats one after the other.
 // What the warp-level kernel needs: two slots per worker of 16 rows x 256 columns.
 constexpr size_t kWarpOnlyWsBytes = kWsPartialOff + (size_t)2 * kMaxWorkers * kWsSlotCols * kMaxSlabM * sizeof(float);

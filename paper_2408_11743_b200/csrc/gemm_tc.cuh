@@ -313,7 +313,8 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
   auto slot_ptr = [&](uint32_t index) { return reinterpret_cast<float4*>(p.partials + (size_t)index * (G::TN * MPAD)); };
   // Blocks x of a tile (x = c32 * nb + b, every `step`-th from x0 on) summed over the slots slot(0) .. slot(n - 1), in order;
   // done(c32, b, f) takes the sums.  Two blocks and two slots at a time: eight 16-byte loads of a lane are in flight together.  What a slot
-  // held is cleared behind its last read: the workspace is zero at rest (but for layers with deferred scales).
+  // held is cleared behind its last read, so that a workspace comes back from most calls as it was given (not with deferred scales, and
+  // not past the last column); nothing relies on it: slots are written before they are read.
   auto sum_blocks = [&](int x0, int step, int items, int nb, uint32_t col, int n, auto slot, auto done) {
     for (int x = x0; x < items; x += 2 * step) {
       int c32[2], b[2];

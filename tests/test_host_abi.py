@@ -179,3 +179,14 @@ def test_no_kernel_of_the_built_library_spills_registers_to_memory():
     assert len(report) >= 20
     bad = {k: v for k, v in report.items() if v[1] > 64}
     assert not bad, bad
+
+
+def test_a_tcgen05_kernel_with_other_registers_fails_the_build():
+    # its launch would be refused (the register split counts on the number): every call would fail instead
+    from paper_2408_11743_b200 import build
+    build.build()
+    report = build.spill_report() or (build.build(force=True), build.spill_report())[1]
+    build.check_registers(report)
+    name = next(k for k in report if "gemm_tc_kernel" in k)
+    with pytest.raises(RuntimeError, match="registers"):
+        build.check_registers({**report, name: (104, 0)})
