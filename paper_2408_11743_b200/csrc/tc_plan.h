@@ -76,9 +76,12 @@ inline TcPlan plan_tc_tile(int nt, int format, int rows, int slabs, int kb, int 
       if (S % d == 0 && S * ncols <= (long long)resident[d] * d) cs = d;
     const long long n = (kb + S - 1) / S;
     static const double placing[9] = {0, 0, 0.13, 0.82, 0.56, 1.29, 1.13, 1.60, 1.40};
+    // large clusters that fill all places of their size start later: 22 of six, 4096 x 2752 with deferred scales at 24 rows 7.1 us
+    // (of four 6.8), groups of 64 rows, 4096 x 5632 at two rows 8.5 (8.0)
+    const bool tight = cs >= 5 && 10 * (S * ncols / cs) > 9 * resident[cs];
     const double fix = S == 1    ? tile
                        : cs == 1 ? exchange * (1.43 + 0.227 * (double)S)
-                                 : exchange + placing[cs] + (S > cs ? 1.46 + exchange * 0.204 * (double)(S / cs) : 0.0);
+                                 : exchange + placing[cs] + (tight ? 0.45 : 0.0) + (S > cs ? 1.46 + exchange * 0.204 * (double)(S / cs) : 0.0);
     take(S * ncols, (int)S, cs, false, per_k_block(S * ncols) * (double)n + fix);
   }
   const long long workers = units < sms ? units : sms;

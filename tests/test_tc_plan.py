@@ -82,6 +82,9 @@ def test_every_plan_can_run(plan, monkeypatch, fmt, env):
     (SPARSE4, 384, 1024, 4096, {(1, 1)}),                  # 7.8 / 6.4
     (SPARSE4, 128, 4096, 4096, {(1, 4), (1, 3)}),          # 10.1 / 9.1
     (DEFERRED4, 160, 1024, 14400, {(1, "whole")}),         # 17.7 / 15.8
+    (DEFERRED4, 24, 4096, 2752, {(1, 4)}),                 # 7.0 in 22 clusters of six / 6.8
+    (DENSE4, 2, 4096, 5632, {(2, 4)}),                     # 8.5 / 8.0, likewise
+    (DEFERRED4, 24, 4096, 1344, {(1, 6)}),                 # half as many clusters of six: 5.7, 6.2 with four
     (ZERO4, 200, 5120, 13824, {(1, "whole")}),             # 42.3 / 38.8 with the k-blocks of DENSE4
     (SPARSE4, 1, 4096, 22016, {(2, "even")}),              # 14.7 / 12.5 with the k-blocks of more rows
     (SPARSE4, 1, 2048, 8192, {(2, 2)}),                    # 6.2 / 5.6
