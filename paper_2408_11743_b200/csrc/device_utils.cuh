@@ -38,6 +38,25 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
+// Have these phases completed?  The tests are issued together, so that their latencies overlap; they do not wait.
+__device__ __forceinline__ bool mbar_test3(uint64_t* a, uint32_t a_parity, uint64_t* b, uint32_t b_parity, uint64_t* c,
+                                           uint32_t c_parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n"
+      ".reg .pred p, q, r;\n"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+      "mbarrier.test_wait.parity.shared::cta.b64 q, [%3], %4;\n"
+      "mbarrier.test_wait.parity.shared::cta.b64 r, [%5], %6;\n"
+      "and.pred p, p, q;\n"
+      "and.pred p, p, r;\n"
+      "selp.u32 %0, 1, 0, p;\n"
+      "}\n"
+      : "=r"(ok)
+      : "r"(smem_u32(a)), "r"(a_parity), "r"(smem_u32(b)), "r"(b_parity), "r"(smem_u32(c)), "r"(c_parity)
+      : "memory");
+  return ok != 0;
+}
 __device__ __forceinline__ uint64_t global_timer_ns() {
   uint64_t t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
@@ -215,6 +234,32 @@ __device__ __forceinline__ void dequant8_biased(uint32_t w, uint32_t (&a)[4]) {
   a[1] = lop3<0xea>(w, HI, EXH);
   a[2] = lop3<0xea>(w2, LO, EXL);
   a[3] = lop3<0xea>(w2, HI, EXH);
+}
+
+// two fp32 values in one 64-bit register pair
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
 }
 
 __device__ __forceinline__ void mma_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {

@@ -80,7 +80,8 @@ struct Geometry {
   // batch rows each.
   static constexpr int CONV_GROUPS = DEF ? 2 : 3, DRAIN_GROUPS = 4 - CONV_GROUPS;
   static constexpr int CONV_WARPS = 4 * CONV_GROUPS, DRAIN_WARPS = 4 * DRAIN_GROUPS;
-  static constexpr int CONV_REGS = DRAIN_GROUPS == 1 ? kLaunchRegs : 88, DRAIN_REGS = DRAIN_GROUPS == 1 ? 152 : 128;
+  static constexpr int CONV_REGS = DRAIN_GROUPS == 1 ? kLaunchRegs : MPAD == 128 ? 80 : 88;
+  static constexpr int DRAIN_REGS = DRAIN_GROUPS == 1 ? 152 : MPAD == 128 ? 136 : 128;
   static_assert(CONV_WARPS * 32 * CONV_REGS + DRAIN_WARPS * 32 * DRAIN_REGS + 128 * kAuxRegs <= kThreads * kLaunchRegs,
                 "setmaxnreg draws on the registers of the launch");
   static constexpr int TN = 128 * NT;
@@ -107,10 +108,13 @@ struct Geometry {
   static constexpr int RING_BYTES = A_STAGES * A_BYTES + W_STAGES * W_BYTES;
   static constexpr int SMEM_BYTES = FIXED_BYTES + 1024 + RING_BYTES;  // 1024: alignment
   // One issuing warp per tile; with one tile the two warps take half of a k-block each, into accumulators of their own that
-  // the drain adds (deferred: whole k-blocks in turn).
+  // the drain adds (deferred: whole k-blocks, in turn or all of them by one warp).
   static constexpr int KH = (DEF || NT == 2) ? 1 : 2;
   static constexpr int STAGE_WARPS = DEF ? 1 : kMmaWarps;     // issuing warps whose commits complete a stage
-  static constexpr int ND = DEF ? (MPAD <= 32 ? 6 : MPAD <= 64 ? 4 : 2) : NT;  // accumulators with a barrier pair of their own
+  // Accumulators with a barrier pair of their own.  Deferred, 128 rows: three of them leave room for two operand slots, which is
+  // the faster split (two and four: the MMAs wait for the read-out; 777 x 4096 x 5504 47.2 us so, 45.0 with three).
+  static constexpr int ND = DEF ? (MPAD <= 32 ? 6 : MPAD <= 64 ? 4 : 3) : NT;
+  static constexpr int ISSUERS = DEF && MPAD == 128 ? 1 : kMmaWarps;  // (an odd ring has one issuer, see the waits)
   static constexpr int D_COLS = DEF ? ND * MPAD : NT * KH * MPAD;
   static constexpr int TILE_A_COLS = SP ? 32 : 64;
   // 2:4: metadata behind the kept values, on even columns (the instruction names a pair of them and which of the two)
@@ -126,7 +130,7 @@ struct Geometry {
   static_assert(SMEM_BYTES <= kSmemBudget, "shared memory");
   static_assert(!DEF || (NT == 1 && FMT == kFmtDense4), "deferred scales: dense, one tile");
   // deferred: each issuer sees its own stages, slots and accumulators
-  static_assert(!DEF || (A_STAGES % 2 == 0 && SLOTS % 2 == 0 && ND % 2 == 0), "the two issuers take the k-blocks in turn");
+  static_assert(!DEF || ISSUERS == 1 || (A_STAGES % 2 == 0 && SLOTS % 2 == 0 && ND % 2 == 0), "the two issuers take the k-blocks in turn");
   // who waits for the MMAs of k-block it - SLOTS knows that those of it - SLOTS - CONV_GROUPS are done (the unit before of the
   // same warpgroup and tile), which has to be past the completion before on the same barrier
   static_assert(A_STAGES >= CONV_GROUPS, "parity of the completion barriers");
@@ -529,12 +533,11 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
       const int mw = warp - kMmaWarp0;
       const int t = NT == 2 ? mw : 0;
       const int h = KH == 2 ? mw : 0;  // half of the k-block
-      // the MMAs of k-block `it` into d_tmem; `fresh`: overwrite what is there
-      auto issue = [&](uint32_t it, uint32_t d_tmem, bool fresh) {
-        const int s = (int)(it % AS), slot = (int)(it % NSLOTS);
+      // the MMAs of the k-block in stage s and operand slot `slot` into d_tmem; `fresh`: overwrite what is there
+      auto issue = [&](uint32_t s, uint32_t slot, uint32_t d_tmem, bool fresh) {
         // descriptor of the first K = 16 step of the stage; the others differ in the address field only
-        const uint64_t desc0 = smem_desc_k_sw128(smem_u32(a_ring) + (uint32_t)s * G::A_BYTES);
-        const uint32_t slot_col = tmem_base + (uint32_t)(G::A_COL0 + slot * G::SLOT_COLS);
+        const uint64_t desc0 = smem_desc_k_sw128(smem_u32(a_ring) + s * (uint32_t)G::A_BYTES);
+        const uint32_t slot_col = tmem_base + (uint32_t)G::A_COL0 + slot * (uint32_t)G::SLOT_COLS;
         const uint32_t a_tmem = slot_col + (uint32_t)(t * G::TILE_A_COLS);
         if constexpr (!SP) {
 #pragma unroll
@@ -556,7 +559,40 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
           }
         }
       };
-      if constexpr (DEF) {
+      if constexpr (DEF && G::ISSUERS == 1) {
+        // Every k-block into the next accumulator of the ring.  The accumulators' round trip (wait, MMAs, completion, read-out,
+        // release) bounds the loop, so the barriers of the next k-block are asked for behind the MMAs of this one, all in one go: one after
+        // the other in front of the MMAs they took 250 cycles.
+        if (mw == 0) {
+          uint32_t s = 0, x_par = 0, slot = 0, a_par = 0, d = 0, d_par = 1;  // (the first filling of an accumulator waits for nothing)
+          bool ready = false;
+          for (uint32_t it = 0; it < total; ++it) {
+            if (!ready) {
+              mbar_wait(&xfull[s], x_par, abort_flag, p.status);
+              mbar_wait(&afull[slot], a_par, abort_flag, p.status);
+              mbar_wait(&dempty[d], d_par, abort_flag, p.status);
+            }
+            tc_fence_after_sync();
+            issue(s, slot, tmem_base + d * (uint32_t)MPAD, true);
+            const uint32_t d_now = d, s_now = s;
+            if (++s == (uint32_t)AS) {
+              s = 0;
+              x_par ^= 1u;
+            }
+            if (++slot == (uint32_t)NSLOTS) {
+              slot = 0;
+              a_par ^= 1u;
+            }
+            if (++d == (uint32_t)G::ND) {
+              d = 0;
+              d_par ^= 1u;
+            }
+            ready = mbar_test3(&xfull[s], x_par, &afull[slot], a_par, &dempty[d], d_par);
+            tc_commit(&dfull[d_now]);
+            tc_commit(&mdone[s_now]);
+          }
+        }
+      } else if constexpr (DEF) {
         // whole k-blocks, the two warps in turn, each into the next accumulator of the ring
         for (uint32_t it = mw; it < total; it += kMmaWarps) {
           const int s = (int)(it % AS), slot = (int)(it % NSLOTS), d = (int)(it % G::ND);
@@ -564,7 +600,7 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
           mbar_wait(&xfull[s], (it / AS) & 1u, abort_flag, p.status);
           mbar_wait(&afull[slot], (it / NSLOTS) & 1u, abort_flag, p.status);
           tc_fence_after_sync();
-          issue(it, tmem_base + (uint32_t)(d * MPAD), true);
+          issue((uint32_t)s, (uint32_t)slot, tmem_base + (uint32_t)(d * MPAD), true);
           tc_commit(&dfull[d]);
           tc_commit(&mdone[s]);
         }
@@ -580,7 +616,7 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
             mbar_wait(&xfull[s], (it / AS) & 1u, abort_flag, p.status);
             mbar_wait(&afull[slot], (it / NSLOTS) & 1u, abort_flag, p.status);
             tc_fence_after_sync();
-            issue(it, d_tmem, x == 0);
+            issue((uint32_t)s, (uint32_t)slot, d_tmem, x == 0);
             // one arrival when these MMAs are done: the slot may be rewritten, the activation tile refilled
             tc_commit(&mdone[s]);
             if (x + 1 == len) tc_commit(&dfull[t]);
@@ -893,9 +929,10 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
       float4* part = p.cluster > 1 ? slot_ptr(worker) : (shared_tile ? stripe_slot((int)worker, vcol) : nullptr);
 
       if constexpr (DEF) {
-        float acc[RBG * 8];
+        // sums of two neighbouring batch rows in a register pair: two rows to an instruction (fma.rn.f32x2)
+        f32x2 acc2[RBG * 4];
 #pragma unroll
-        for (int e = 0; e < RBG * 8; ++e) acc[e] = 0.f;
+        for (int e = 0; e < RBG * 4; ++e) acc2[e] = pack2(0.f, 0.f);
         // the scales of a k-block, loaded (from the L2, see above) while the one before is added
         auto load_scale = [&](uint32_t x) {
           uint2 v = make_uint2(0, 0);
@@ -911,11 +948,12 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
           const int d = (int)(it % G::ND);
           const float2 s01 = __half22float2(*reinterpret_cast<const __half2*>(&sv.x));
           const float2 s23 = __half22float2(*reinterpret_cast<const __half2*>(&sv.y));
+          const f32x2 sc2[4] = {pack2(s01.x, s01.x), pack2(s01.y, s01.y), pack2(s23.x, s23.x), pack2(s23.y, s23.y)};
           sv = load_scale(x + 1);
           mbar_wait(&dfull[d], (it / G::ND) & 1u, abort_flag, p.status);
           tc_fence_after_sync();
-          // (64 rows of a warpgroup: 16 at a time, to spare registers)
-          constexpr int MG = RBG * 8, MC = MG > 32 ? 16 : MG;
+          // (64 rows of a warpgroup: 32 at a time, to spare registers)
+          constexpr int MG = RBG * 8, MC = imin(MG, 32);
 #pragma unroll
           for (int m0 = 0; m0 < MG; m0 += MC) {
             float dd[MC / 16][2][8];
@@ -931,13 +969,16 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
 #pragma unroll
               for (int h = 0; h < 2; ++h)
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                  const float sc = h == 0 ? ((e & 2) ? s01.y : s01.x) : ((e & 2) ? s23.y : s23.x);
-                  float& a = acc[(m0 / 8 + b) * 8 + 4 * h + e];
-                  a = fmaf(sc, dd[b >> 1][h][4 * (b & 1) + e], a);
+                for (int e = 0; e < 2; ++e) {
+                  const float* v = &dd[b >> 1][h][4 * (b & 1) + 2 * e];
+                  f32x2& a = acc2[(m0 / 8 + b) * 4 + 2 * h + e];
+                  a = fma2(sc2[2 * h + e], pack2(v[0], v[1]), a);
                 }
           }
         }
+        float acc[RBG * 8];
+#pragma unroll
+        for (int e = 0; e < RBG * 4; ++e) unpack2(acc2[e], acc[2 * e], acc[2 * e + 1]);
         before_first_write();
         if (part) {
 #pragma unroll

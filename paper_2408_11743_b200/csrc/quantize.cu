@@ -23,6 +23,7 @@
 // for the error) and two comparisons beside it; rintf() would be a conversion instruction at an eighth of the rate, and
 // was what bounded this file before.  The operations are issued on pairs (fma.rn.f32x2 and the like: the same
 // IEEE operations, half the instructions).
+#include "device_utils.cuh"
 #include "marlin_internal.cuh"
 
 namespace marlin_b200 {
@@ -30,31 +31,6 @@ namespace {
 
 __device__ __forceinline__ float load_w(const uint16_t* p) { return __half2float(__ushort_as_half(__ldg(p))); }
 
-// two fp32 values in one 64-bit register pair
-typedef unsigned long long f32x2;
-__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
-  f32x2 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ void unpack2(f32x2 v, float& lo, float& hi) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
-  f32x2 r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
-  f32x2 r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
-  f32x2 r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
 __device__ __forceinline__ f32x2 clamp2(f32x2 x) {
   float lo, hi;
   unpack2(x, lo, hi);
