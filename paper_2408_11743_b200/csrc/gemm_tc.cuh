@@ -14,7 +14,8 @@
 //                 (Section 3.4 "Dequantization and Tensor Cores") and writes them into an operand slot with tcgen05.st
 //                 (64 columns, two k per column).
 //   warps 12..15  drain (8..15 with deferred scales): accumulators out of tensor memory, fix-up across CTAs, C.  They have
-//                 no part in the conversion, so the next column segment is converted meanwhile.
+//                 no part in the conversion, so the next column segment is converted meanwhile.  The last tile of a CTA is read
+//                 out by the converters as well (not with deferred scales, whose sums are in the drain's registers).
 //   warp 16       weight producer: one bulk copy of packed weights per k-block (evict-first) into a ring that the converters
 //                 free.
 //   warp 17       activation producer: per k-block one TMA box (two 64-wide halves, 128-byte swizzle = the canonical K-major
@@ -214,6 +215,7 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
   uint32_t* tmem_base_slot = reinterpret_cast<uint32_t*>(smem + 832);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + 836);
   volatile int* last_flag = reinterpret_cast<volatile int*>(smem + 840);
+  volatile int* others_flag = reinterpret_cast<volatile int*>(smem + 844);  // the others have left their parts of the last tile
   uint8_t* a_ring = smem + G::FIXED_BYTES;
   uint8_t* w_ring = a_ring + AS * G::A_BYTES;
 
@@ -453,6 +455,181 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
     }
   };
 
+  // ---- read-out of accumulators: used by the drain and, for a CTA's last tile, by the converters too ----
+  const uint32_t quad = (uint32_t)(warp & 3);  // 32 TMEM lanes = channels of a tile
+  // the scales of channels lane / 4, +8, +16, +24 of the warp's 32 are four halves in a row
+  const uint32_t spos2 = ((quad >> 1) * 64 + 8 * (uint32_t)(lane >> 2) + 4 * (quad & 1)) * 2;
+  auto column_scales = [&](uint32_t col, int t, float (&sc)[4]) {
+    sc[0] = sc[1] = sc[2] = sc[3] = 1.f;
+    if constexpr (SCALE == kPerColumn) {
+      uint2 sv = make_uint2(0, 0);
+      if (col * G::TN + (uint32_t)t * 128 + quad * 32 < (uint32_t)p.N)
+        sv = __ldg(reinterpret_cast<const uint2*>(p.sq + ((size_t)col * G::TN + (size_t)t * 128) * 2 + spos2));
+      const float2 s01 = __half22float2(*reinterpret_cast<const __half2*>(&sv.x));
+      const float2 s23 = __half22float2(*reinterpret_cast<const __half2*>(&sv.y));
+      sc[0] = s01.x; sc[1] = s01.y; sc[2] = s23.x; sc[3] = s23.y;
+    }
+  };
+  // 16 rows from row m on out of tensor memory, the halves of the k-blocks added, scaled: f[8b + 4h + e]
+  auto load_rows = [&](int t, int m, const float (&sc)[4], float (&f)[16]) {
+    float a[2][8], a2[2][8];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const uint32_t at = tmem_base + ((quad * 32u + (uint32_t)(16 * h)) << 16) + (uint32_t)(t * KH * MPAD + m);
+      tc_ld_frag(at, a[h]);
+      if constexpr (KH == 2) tc_ld_frag(at + MPAD, a2[h]);
+    }
+    tc_wait_ld();
+#pragma unroll
+    for (int x = 0; x < 16; ++x) {
+      const int h = (x >> 2) & 1, i = 4 * (x >> 3) + (x & 3);
+      f[x] = a[h][i];
+      if constexpr (KH == 2) f[x] += a2[h][i];
+      if constexpr (SCALE == kPerColumn) f[x] *= sc[2 * h + ((x >> 1) & 1)];
+    }
+  };
+  // The CTA's last tile (not with deferred scales): the converters have nothing else left to do, so all 16 warps read it out, in pieces
+  // of 16 rows x 32 channels; piece c: tile c % NT, rows 16 (c / NT).  With the four draining warps alone this took 0.55 us (32 rows,
+  // two tiles) to 2.1 us (128 rows) at the end of every launch.
+  auto drain_last = [&](int w16) {
+    const uint32_t vcol = (u1 - 1) / KB, col = vcol / p.slabs, slab = vcol - col * p.slabs;
+    const uint32_t phase = (vcol - u0 / KB) & 1u;
+    const size_t row0 = (size_t)slab * MPAD;
+    const int m_lim = min(p.M - (int)row0, MPAD);
+    const int pieces = NT * ((m_lim + 15) >> 4), g = w16 >> 2;
+    const int first_w = p.split ? (int)(vcol * p.split) : (int)stripe_owner32(vcol * KB, U, P);
+    const int last_w = p.split ? (int)(vcol * p.split + p.split - 1) : (int)stripe_owner32((vcol + 1) * KB - 1, U, P);
+    const bool shared_tile = !p.whole && last_w > first_w, clustered = p.cluster > 1;
+    int* stripe_counter = &p.counters[(uint32_t)p.ncols <= P ? vcol : (uint32_t)first_w];
+    // what is in tensor memory of piece c
+    auto own_sums = [&](int c, float (&f)[16]) {
+      const int t = c % NT;
+      float sc[4];
+      column_scales(col, t, sc);
+      mbar_wait(&dfull[t], phase, abort_flag, p.status);
+      tc_fence_after_sync();
+      load_rows(t, c / NT * 16, sc, f);
+    };
+    // block y / 2 of the piece (rows), half y % 2 (channels), in a slot
+    auto piece_index = [&](int c, int y) { return frag_index((c % NT) * 4 + (int)quad, c / NT * 2 + (y >> 1), y & 1); };
+    auto in_rows = [&](int c, int y) { return c / NT * 16 + 8 * (y >> 1) < m_lim; };
+    auto to_slot = [&](int c, const float (&f)[16], float4* slot) {
+#pragma unroll
+      for (int y = 0; y < 4; ++y)
+        if (in_rows(c, y)) slot[piece_index(c, y)] = make_float4(f[4 * y], f[4 * y + 1], f[4 * y + 2], f[4 * y + 3]);
+    };
+    auto to_c = [&](int c, const float (&f)[16]) {
+      const int c32 = (c % NT) * 4 + (int)quad;
+      if (col * G::TN + (uint32_t)c32 * 32 >= (uint32_t)p.N) return;
+#pragma unroll
+      for (int b = 0; b < 2; ++b) {
+        float fb[8];
+#pragma unroll
+        for (int x = 0; x < 8; ++x) fb[x] = f[8 * b + x];
+        store_block(c32, c / NT * 2 + b, fb, b, col, m_lim, row0);
+      }
+    };
+    // Piece c of n partial tiles in their order: tile `own` (n: none) from tensor memory, the others from their slots, two of them on
+    // their way at a time, and cleared behind the read (a workspace comes back as it was given).
+    auto gather = [&](int c, int n, int own, auto slot, float (&sum)[16]) {
+      float f[16];
+      if (own < n) own_sums(c, f);
+#pragma unroll
+      for (int x = 0; x < 16; ++x) sum[x] = 0.f;
+      const int others = own < n ? n - 1 : n;
+      for (int o = 0; o < others; o += 2) {
+        float4 v[2][4];
+        float4* from[2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+          if (o + i < others) {
+            from[i] = slot(o + i + (o + i >= own ? 1 : 0));
+#pragma unroll
+            for (int y = 0; y < 4; ++y)
+              if (in_rows(c, y)) v[i][y] = ld_cg_f4(from[i] + piece_index(c, y));
+          }
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+          if (o + i < others) {
+            if (o + i == own) {
+#pragma unroll
+              for (int x = 0; x < 16; ++x) sum[x] += f[x];
+            }
+#pragma unroll
+            for (int y = 0; y < 4; ++y)
+              if (in_rows(c, y)) {
+                sum[4 * y] += v[i][y].x; sum[4 * y + 1] += v[i][y].y; sum[4 * y + 2] += v[i][y].z; sum[4 * y + 3] += v[i][y].w;
+                from[i][piece_index(c, y)] = make_float4(0.f, 0.f, 0.f, 0.f);
+              }
+          }
+      }
+      if (own == n - 1) {
+#pragma unroll
+        for (int x = 0; x < 16; ++x) sum[x] += f[x];
+      }
+    };
+    pdl_wait_prior_grids();
+    float f[16];
+    if (clustered) {
+      // CTAs of a split tile in clusters: the pieces are dealt out to them.  A CTA leaves those of the others in its slot and, behind the
+      // cluster barrier, adds the others' parts of its own pieces to what it has in tensor memory, in rank order.  (Through the L2 and not
+      // through distributed shared memory: bulk copies from one shared memory into another, which exchange 32 KB among four CTAs in 2630
+      // cycles instead of 4170, need a handshake before them and a barrier before a CTA may exit, and took 1 to 1.5 us longer in all.)
+      const int cs = (int)p.cluster, C = (int)p.split / cs, r = (int)cluster_ctarank();
+      float4* mine = slot_ptr(worker);
+      for (int c = g; c < pieces; c += 4)
+        if (c % cs != r) {
+          own_sums(c, f);
+          to_slot(c, f, mine);
+        }
+      cluster_sync_all();
+      const uint32_t first = worker - (uint32_t)r, shares = P + vcol * (uint32_t)C;
+      for (int c = r + cs * g; c < pieces; c += 4 * cs) {
+        gather(c, cs, r, [&](int q) { return slot_ptr(first + (uint32_t)q); }, f);
+        if (C == 1)
+          to_c(c, f);
+        else
+          to_slot(c, f, slot_ptr(shares + (worker / (uint32_t)cs) % (uint32_t)C));
+      }
+      if (C == 1) return;
+      // the CTAs of rank r of the tile's clusters hold the same pieces: whoever of them comes last adds them up
+      named_bar_sync(1, kAuxWarp0 * 32);
+      if (w16 == 0 && lane == 0) {
+        int* counter = &p.counters[vcol * (uint32_t)cs + r];
+        const int is_last = atom_add_acq_rel_gpu(counter, 1) == C - 1 ? 1 : 0;
+        if (is_last) *counter = 0;
+        *last_flag = is_last;
+      }
+      named_bar_sync(1, kAuxWarp0 * 32);
+      if (*last_flag != 0)
+        for (int c = r + cs * g; c < pieces; c += 4 * cs) {
+          gather(c, C, C, [&](int q) { return slot_ptr(shares + (uint32_t)q); }, f);
+          to_c(c, f);
+        }
+      return;
+    }
+    // Stripes.  Where the other CTAs of the tile have left their parts already (the usual case: it was their first tile), this one adds
+    // them to what it has and writes C; otherwise it leaves its own, and the last arriver adds up all of them.
+    if (w16 == 0 && lane == 0) *others_flag = shared_tile && ld_acquire_gpu(stripe_counter) == last_w - first_w ? 1 : 0;
+    named_bar_sync(1, kAuxWarp0 * 32);  // (also: the drain is done with the tile before, which went through all output buffers)
+    const bool onto = *others_flag != 0;
+    for (int c = g; c < pieces; c += 4) {
+      if (onto)
+        gather(c, last_w - first_w + 1, (int)worker - first_w, [&](int q) { return stripe_slot(first_w + q, vcol); }, f);
+      else
+        own_sums(c, f);
+      if (shared_tile && !onto)
+        to_slot(c, f, stripe_slot((int)worker, vcol));
+      else
+        to_c(c, f);
+    }
+    if (onto) {
+      if (w16 == 0 && lane == 0) *stripe_counter = 0;
+    } else {
+      finish_stripe(w16);
+    }
+  };
+
   if (warp >= kAuxWarp0) {
     setmaxnreg_dec<kAuxRegs>();
     if (warp == kWeightWarp) {
@@ -627,7 +804,8 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
     }
     __syncwarp();
     if (p.cluster > 1) cluster_sync_all();  // every thread of every CTA of the cluster takes part
-  } else if (warp < G::CONV_WARPS) {
+  } else {  // converters and drain: two roles with one end
+  if (warp < G::CONV_WARPS) {
     // --------------------------------- converters ------------------------------------------------------------------
     if constexpr (G::CONV_REGS < kLaunchRegs) setmaxnreg_dec<G::CONV_REGS>();
     const uint32_t wg = (uint32_t)(warp >> 2);
@@ -823,10 +1001,6 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
         convert_all(BoolC<false>{}, sq, zq4);
       }
     }
-    if (p.cluster > 1)
-      finish_cluster(warp);
-    else
-      finish_stripe(warp);
   } else {
     // --------------------------------- drain: accumulators, fix-up, C ----------------------------------------------
     setmaxnreg_inc<G::DRAIN_REGS>();
@@ -836,8 +1010,6 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
     const int b_first = (warp - G::CONV_WARPS) / 4 * RBG;
     const uint32_t tmem_lane = tmem_base + ((uint32_t)dw * 32u << 16);  // this warp's TMEM lanes = channels of a tile
     const int dtid = (int)threadIdx.x - G::CONV_WARPS * 32;
-    // the scales of channels lane / 4, +8, +16, +24 of the warp's 32 are four halves in a row
-    const uint32_t spos2 = (uint32_t)((dw >> 1) * 64 + 8 * (lane >> 2) + 4 * (dw & 1)) * 2;
     auto release = [&](int d) {
       tc_fence_before_sync();
       __syncwarp();
@@ -925,6 +1097,7 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
           if (zp) asm volatile("prefetch.global.L2 [%0];" ::"l"(p.zq + at * 2));
         }
       }
+      if (!DEF && u + len == u1) break;  // the last tile: drain_last
       // where the partial tile goes, if this is one
       float4* part = p.cluster > 1 ? slot_ptr(worker) : (shared_tile ? stripe_slot((int)worker, vcol) : nullptr);
 
@@ -1004,42 +1177,17 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
       } else {
 #pragma unroll 1
         for (int t = 0; t < NT; ++t) {
-          float sc[4] = {1.f, 1.f, 1.f, 1.f};
+          float sc[4];
           const uint32_t n0 = ncol0 + (uint32_t)t * 128;
-          if constexpr (SCALE == kPerColumn) {
-            uint2 sv = make_uint2(0, 0);
-            if (n0 < (uint32_t)p.N)
-              sv = __ldg(reinterpret_cast<const uint2*>(p.sq + ((size_t)col * G::TN + (size_t)t * 128) * 2 + spos2));
-            const float2 s01 = __half22float2(*reinterpret_cast<const __half2*>(&sv.x));
-            const float2 s23 = __half22float2(*reinterpret_cast<const __half2*>(&sv.y));
-            sc[0] = s01.x; sc[1] = s01.y; sc[2] = s23.x; sc[3] = s23.y;
-          }
+          column_scales(col, t, sc);
           before_first_write();
           mbar_wait(&dfull[t], seg & 1u, abort_flag, p.status);
           tc_fence_after_sync();
-          // 16 rows from row m on out of tensor memory, the halves of the k-blocks added, scaled: f[8b + 4h + e]
-          auto load_rows = [&](int m, float (&f)[16]) {
-            float a[2][8], a2[2][8];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              const uint32_t at = tmem_lane + ((uint32_t)(16 * h) << 16) + (uint32_t)(t * KH * MPAD + m);
-              tc_ld_frag(at, a[h]);
-              if constexpr (KH == 2) tc_ld_frag(at + MPAD, a2[h]);
-            }
-            tc_wait_ld();
-#pragma unroll
-            for (int x = 0; x < 16; ++x) {
-              const int h = (x >> 2) & 1, i = 4 * (x >> 3) + (x & 3);
-              f[x] = a[h][i];
-              if constexpr (KH == 2) f[x] += a2[h][i];
-              if constexpr (SCALE == kPerColumn) f[x] *= sc[2 * h + ((x >> 1) & 1)];
-            }
-          };
           if (part) {
 #pragma unroll 2
             for (int m = 0; m < MPAD; m += 16) {
               float f[16];
-              load_rows(m, f);
+              load_rows(t, m, sc, f);
               if (m + 16 == MPAD) release(t);
 #pragma unroll
               for (int b = 0; b < 2; ++b)
@@ -1057,7 +1205,7 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
 #pragma unroll
             for (int m = 0; m < MPAD; m += 16) {
               float f[16];
-              load_rows(m, f);
+              load_rows(t, m, sc, f);
 #pragma unroll
               for (int b = 0; b < 2; ++b) {
                 const int x = m / 8 + b;
@@ -1107,14 +1255,20 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
       }
       u += len;
     }
-    if (p.cluster > 1)
-      finish_cluster(warp);
-    else
-      finish_stripe(warp);
-    if (*abort_flag) {
-      // a wait gave up: copies may still be in flight towards this CTA's shared memory
-      for (int x = 0; x < 1000; ++x) __nanosleep(1000);
-    }
+    setmaxnreg_dec<G::CONV_REGS>();  // what follows is the converters' code as well
+  }
+
+  // --------------------------------- the end of the CTA's last tile ----------------------------------------------
+  if constexpr (!DEF)
+    drain_last(warp);
+  else if (p.cluster > 1)
+    finish_cluster(warp);
+  else
+    finish_stripe(warp);
+  if (*abort_flag) {
+    // a wait gave up: copies may still be in flight towards this CTA's shared memory
+    for (int x = 0; x < 1000; ++x) __nanosleep(1000);
+  }
   }
 
   // ---- the TMEM owner waits for everybody who touches tensor memory, then frees it ----
