@@ -5,7 +5,7 @@
 // architecture.  Here the product is computed transposed, as the paper does for its sparse kernel (Section 4:
 // C = (B^T A^T)^T): per column tile of W and 128-row k-block
 //     D_t[128 channels x MPAD batch rows] += W_t^T[128 x 128] . A^T[128 x MPAD],   t = 0 .. NT - 1
-// with UMMA shape M = 128 (output channels on the TMEM lanes), N = MPAD (batch), K = 16.
+// with UMMA shape M = 128 (output channels on the TMEM lanes), N = the rows of a slab (at most MPAD), K = 16.
 //
 // One CTA per SM, 640 threads:
 //   warps 0..11   converters, three warpgroups (two with deferred scales) that take the k-blocks in turn: one converts while
@@ -86,8 +86,7 @@ struct Geometry {
   static_assert(CONV_WARPS * 32 * CONV_REGS + DRAIN_WARPS * 32 * DRAIN_REGS + 128 * kAuxRegs <= kThreads * kLaunchRegs,
                 "setmaxnreg draws on the registers of the launch");
   static constexpr int TN = 128 * NT;
-  static constexpr int A_HALF_BYTES = MPAD * 128;
-  static constexpr int A_BYTES = 2 * A_HALF_BYTES;
+  static constexpr int A_BYTES = MPAD * 256;
   static constexpr int CODE_BYTES = SP ? TN * 32 : (W8 ? TN * 128 : TN * 64);
   static constexpr int META_BYTES = SP ? TN * 16 : 0;
   static constexpr int W_BYTES = CODE_BYTES + META_BYTES;
@@ -235,6 +234,8 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
                       : p.whole ? stripe_begin32(worker + 1, (uint32_t)p.ncols, P) * KB
                                 : stripe_begin32(worker + 1, U, P);
   const uint32_t total = u1 - u0;  // k-blocks of this CTA
+  // Rows of a slab: a multiple of 16, at most MPAD.  (Deferred scales: always MPAD, see tc_slab_rows.)
+  const uint32_t slab_rows = DEF ? (uint32_t)MPAD : p.slab_rows;
   const bool zp = SCALE != kPerColumn && p.zq != nullptr;  // zero points: rows of the same shape and order as the scales
 
   pdl_launch_dependents();
@@ -396,8 +397,8 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
   auto finish_cluster = [&](int w16) {
     const int cs = (int)p.cluster, C = (int)p.split / cs, r = (int)cluster_ctarank();
     const uint32_t vcol = u0 / KB, col = vcol / p.slabs, slab = vcol - col * p.slabs;
-    const size_t row0 = (size_t)slab * MPAD;
-    const int m_lim = min(p.M - (int)row0, MPAD);
+    const size_t row0 = (size_t)slab * slab_rows;
+    const int m_lim = min(p.M - (int)row0, (int)slab_rows);
     const int nb = (m_lim + 7) >> 3, items = nb * (G::TN / 32);
     cluster_sync_all();  // every CTA's partial tile is in its slot
     if (w16 < G::CONV_WARPS) pdl_wait_prior_grids();
@@ -438,8 +439,8 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
     const int last_w = p.split ? (int)(vcol * p.split + p.split - 1) : (int)stripe_owner32((vcol + 1) * KB - 1, U, P);
     if (p.whole || last_w == first_w) return;
     if (w16 < G::CONV_WARPS) pdl_wait_prior_grids();
-    const size_t row0 = (size_t)slab * MPAD;
-    const int m_lim = min(p.M - (int)row0, MPAD);
+    const size_t row0 = (size_t)slab * slab_rows;
+    const int m_lim = min(p.M - (int)row0, (int)slab_rows);
     const int nb = (m_lim + 7) >> 3, items = nb * (G::TN / 32);
     named_bar_sync(1, kAuxWarp0 * 32);
     if (w16 == 0 && lane == 0) {
@@ -494,8 +495,8 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
   auto drain_last = [&](int w16) {
     const uint32_t vcol = (u1 - 1) / KB, col = vcol / p.slabs, slab = vcol - col * p.slabs;
     const uint32_t phase = (vcol - u0 / KB) & 1u;
-    const size_t row0 = (size_t)slab * MPAD;
-    const int m_lim = min(p.M - (int)row0, MPAD);
+    const size_t row0 = (size_t)slab * slab_rows;
+    const int m_lim = min(p.M - (int)row0, (int)slab_rows);
     const int pieces = NT * ((m_lim + 15) >> 4), g = w16 >> 2;
     const int first_w = p.split ? (int)(vcol * p.split) : (int)stripe_owner32(vcol * KB, U, P);
     const int last_w = p.split ? (int)(vcol * p.split + p.split - 1) : (int)stripe_owner32((vcol + 1) * KB - 1, U, P);
@@ -692,8 +693,8 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
         for (uint32_t it = 0; it < total; ++it) {
           const uint32_t s = it % AS;
           if (it >= (uint32_t)AS) mbar_wait<20>(&mdone[s], (it / AS - 1) & 1u, abort_flag, p.status);
-          mbar_expect_tx(&xfull[s], G::A_BYTES);
-          tma_load_3d(a_ring + (size_t)s * G::A_BYTES, &tmap_a, 0, (int)(slab * MPAD), (int)(2 * kb), &xfull[s], pol_a);
+          mbar_expect_tx(&xfull[s], slab_rows * 256u);
+          tma_load_3d(a_ring + (size_t)s * G::A_BYTES, &tmap_a, 0, (int)(slab * slab_rows), (int)(2 * kb), &xfull[s], pol_a);
           if (++kb == KB) {
             kb = 0;
             if (++slab == p.slabs) slab = 0;
@@ -705,7 +706,8 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
       }
     } else if (elect_one()) {
       // ------------------------------- MMA issuers (one thread each) -------------------------------------------------
-      constexpr uint32_t idesc = instr_desc_f16(128, MPAD);
+      // N: the rows of a slab; the halves of an activation tile lie that many rows apart
+      const uint32_t idesc = instr_desc_f16(128, (int)slab_rows), half_step = slab_rows * 8u;
       constexpr int KS = 8 / KH;  // K = 16 steps per warp and k-block
       const int mw = warp - kMmaWarp0;
       const int t = NT == 2 ? mw : 0;
@@ -720,7 +722,7 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
 #pragma unroll
           for (int k2 = 0; k2 < KS; ++k2) {
             const int ks = h * KS + k2;
-            const uint64_t bdesc = desc0 + (uint64_t)(((ks >> 2) * G::A_HALF_BYTES + (ks & 3) * 32) >> 4);
+            const uint64_t bdesc = desc0 + (uint64_t)((ks >> 2) * half_step + (ks & 3) * 2);
             tc_mma_ts(d_tmem, a_tmem + ks * 8, bdesc, idesc, (fresh && k2 == 0) ? 0u : 1u);
           }
         } else {
@@ -730,7 +732,7 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
 #pragma unroll
           for (int k2 = 0; k2 < KS / 2; ++k2) {
             const int i = h * (KS / 2) + k2;
-            const uint64_t bdesc = desc0 + (uint64_t)(((i >> 1) * G::A_HALF_BYTES + (i & 1) * 64) >> 4);
+            const uint64_t bdesc = desc0 + (uint64_t)((i >> 1) * half_step + (i & 1) * 4);
             tc_mma_sp_ts(d_tmem, a_tmem + i * 8, bdesc, e_tmem + (uint32_t)(i & ~1), idesc | kIdescSparse | (uint32_t)(i & 1),
                          (fresh && k2 == 0) ? 0u : 1u);
           }
@@ -1059,12 +1061,12 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
     uint32_t it = 0, seg = 0;
     bool waited_for_prior_grid = false;
     for (uint32_t u = u0; u < u1; ++seg) {
-      // virtual column tile = (column tile of W, slab of MPAD batch rows): batches above MPAD rows replicate the
+      // virtual column tile = (column tile of W, slab of batch rows): batches above MPAD rows replicate the
       // layer in the unit numbering (Section 3.4, last paragraph), slab after slab of one column tile
       const uint32_t vcol = u / KB;
       const uint32_t col = vcol / p.slabs, slab = vcol - col * p.slabs;
-      const size_t row0 = (size_t)slab * MPAD;
-      const int m_lim = min(p.M - (int)row0, MPAD);  // rows of this slab that exist
+      const size_t row0 = (size_t)slab * slab_rows;
+      const int m_lim = min(p.M - (int)row0, (int)slab_rows);  // rows of this slab that exist
       const uint32_t len = min(KB - u % KB, u1 - u);
       const uint32_t ncol0 = col * G::TN + (uint32_t)dw * 32;  // first channel of this warp in tile 0
       const int first_w = p.split ? (int)(vcol * p.split) : (int)stripe_owner32(vcol * KB, U, P);
@@ -1299,7 +1301,7 @@ cudaError_t launch(const GemmParams& p, cudaStream_t stream) {
     if (dev >= 0 && dev < 64) attr_set[dev] = true;
   }
   alignas(64) CUtensorMap tmap;
-  if (!make_a_tensor_map_3d(&tmap, p.A, p.M, p.K, MPAD)) return cudaErrorInvalidValue;
+  if (!make_a_tensor_map_3d(&tmap, p.A, p.M, p.K, (int)p.slab_rows)) return cudaErrorInvalidValue;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(workers);
   cfg.blockDim = dim3(kThreads);

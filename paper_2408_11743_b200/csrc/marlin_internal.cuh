@@ -84,8 +84,9 @@ struct GemmParams {
   uint32_t team_tiles, team_extra;  // warp-MMA kernel, split > 0: column tiles per team; teams with one more
   uint32_t cluster;  // warp-MMA kernel: 1, 2, 3 = the CTAs of a team form a cluster (see there); tcgen05 kernel: CTAs per
                      // cluster (a divisor of `split`; 0, 1: none)
-  uint32_t slabs;    // tcgen05 kernel: slabs of batch rows (32, 64 or 128) in this launch; virtual column tile
+  uint32_t slabs;    // tcgen05 kernel: slabs of batch rows in this launch; virtual column tile
                      // v = column tile v / slabs of W, rows of slab v % slabs
+  uint32_t slab_rows;  // tcgen05 kernel: rows of a slab (tc_slab_rows): a multiple of 16, at most 32, 64 or 128 (the instance's)
   uint32_t whole;    // tcgen05 kernel: 1 = worker w owns the virtual column tiles [w * ncols / P, (w + 1) * ncols / P) whole
   uint32_t split;    // tcgen05 kernel: 0 = even stripes over all units; S > 0 = every column tile is cut into S
                      // k-ranges and worker w owns range w % S of tile w / S (one segment per CTA)

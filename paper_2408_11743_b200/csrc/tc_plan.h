@@ -11,6 +11,15 @@ enum TcFormat { kTcDense4 = 0, kTcSparse4 = 1, kTcDense8 = 2, kTcDeferred4 = 3, 
 // rows of a slab: the MMA's N
 inline int tc_mpad(int m) { return m <= 32 ? 32 : (m <= 64 ? 64 : 128); }
 
+// Batches are cut into equal slabs, in units of 16 rows: what MMAs, copies and read-out cost goes with the rows of a slab, so 130 rows are two
+// slabs of 80, not of 128 (8192 x 8192 at 130 rows 25.1 us so, 24.1 now; 4096 x 22016 at 100 rows 25.6 / 24.6; 2:4, 4096 x 4096 at 300 rows
+// 12.6 / 12.2).  With deferred scales the round trip of the accumulators bounds the loop, and an issuer that reads the rows at run time
+// makes it longer: those slabs are whole (128 rows of 4096 x 5504 12.2 us, 12.6 with the same rows at run time).
+inline int tc_slab_rows(int format, int m) {
+  const int mpad = tc_mpad(m), slabs = (m + mpad - 1) / mpad;
+  return format == kTcDeferred4 ? mpad : ((m + slabs - 1) / slabs + 15) / 16 * 16;
+}
+
 struct TcPlan {
   int nt;                     // 128-column UMMA tiles per CTA
   long long ncols, workers;   // (column tile, slab) pairs; CTAs
@@ -91,7 +100,7 @@ inline TcPlan plan_tc_tile(int nt, int format, int rows, int slabs, int kb, int 
     if (contributors < 2.0) contributors = 2.0;
     double far = 0.0;
     if (slabs > 1 && nt == 1) {
-      far = ((double)slabs * mpad * kb * 256.0 - 40e6) / 40e6;
+      far = ((double)slabs * rows * kb * 256.0 - 40e6) / 40e6;
       far = far < 0.0 ? 0.0 : far > 1.0 ? 1.0 : far;
     }
     take(workers, 0, 0, false,
@@ -107,11 +116,12 @@ inline TcPlan plan_tc_tile(int nt, int format, int rows, int slabs, int kb, int 
 // M rows on a layer of N columns and kb k-blocks; deferred scales have tiles of 128 columns alone
 inline TcPlan plan_tc(int format, int M, int kb, int N, int sm_count, int max_workers) {
   const int mpad = tc_mpad(M), slabs = (M + mpad - 1) / mpad;
+  const int rows = slabs == 1 ? M : tc_slab_rows(format, M);
   const char* columns = getenv("MARLIN_B200_TC_TILE");  // tuning knob: 128 or 256 columns per tile, where there is a choice
   TcPlan best{};
   for (int nt = 1; nt <= 2; ++nt) {
     if (format == kTcDeferred4 ? nt != 1 : (columns && (atoi(columns) == 128) != (nt == 1))) continue;
-    const TcPlan p = plan_tc_tile(nt, format, M < mpad ? M : mpad, slabs, kb, N, sm_count, max_workers);
+    const TcPlan p = plan_tc_tile(nt, format, rows, slabs, kb, N, sm_count, max_workers);
     if (!best.nt || p.cost < best.cost) best = p;
   }
   return best;

@@ -49,6 +49,23 @@ def test_integer_closed_form_is_bit_exact_above_128_rows(marlin, oracle_lib, mon
 
 
 @pytest.mark.parametrize("mode", range(len(MODES)))
+@pytest.mark.parametrize("M", [1, 16, 17, 33, 48, 49, 65, 80, 81, 112, 113, 129, 130, 160, 161, 224, 225, 257, 384, 385, 777])
+def test_slabs_of_every_height_are_bit_exact(marlin, oracle_lib, monkeypatch, mode, M):
+    # the rows of a slab are a multiple of 16 that depends on the batch; groups of 64 rows: the tcgen05 kernel at every batch size.
+    # Sums of small integers and powers of two: exact in fp32 in any order.
+    for k, v in MODES[mode].items():
+        monkeypatch.setenv(k, v)
+    K, N, G = 640, 768, 64
+    rng = np.random.default_rng(M)
+    Q = rng.integers(0, 16, size=(K, N), dtype=np.uint8)
+    A = rng.integers(-3, 4, size=(M, K)).astype(np.float16)
+    S = np.ldexp(1.0, rng.integers(-4, 1, size=(K // G, N))).astype(np.float16)
+    q = inputs.kpack(Q)
+    C = DenseLayer(marlin, q, S, G, max_M=M)(A)
+    assert np.array_equal(C.view(np.uint16), oracle_lib.gemm(A, q, S, G).view(np.uint16))
+
+
+@pytest.mark.parametrize("mode", range(len(MODES)))
 def test_unit_vectors_reach_every_slab_and_k_position(marlin, monkeypatch, mode):
     # row m is the unit vector of k = (37 m) mod K: C[m, n] = (Q[k, n] - 8) * S[k / G, n] exactly
     for k, v in MODES[mode].items():
