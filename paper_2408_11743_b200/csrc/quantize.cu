@@ -16,13 +16,19 @@
 // what runs in parallel.
 //   - Groups of 32, 64 or 128 rows: one thread owns one (group, column) and holds its rows in registers, one read of W.
 //   - Longer groups (up to one scale per column): three launches.  Column maxima in parts of 128 rows; then the search
-//     with one thread per (column, pair of candidates), so that the serial sum over the rows runs for all candidates at
+//     with one thread per (column, candidate), so that the serial sum over the rows runs for all candidates at
 //     once; then the codes, parallel over the rows.  (One thread per column, which re-read the group once per candidate,
-//     left the chip idle on such layers: 4096 x 4096 with one scale per column took 7.96 ms; 100 us now.)
-// Bound: the fp32 pipe.  Per weight and candidate there are five operations on it (product, two for the rounding, two
-// for the error) and two comparisons beside it; rintf() would be a conversion instruction at an eighth of the rate, and
-// was what bounded this file before.  The operations are issued on pairs (fma.rn.f32x2 and the like: the same
-// IEEE operations, half the instructions).
+//     left the chip idle on such layers: 4096 x 4096 with one scale per column took 7.96 ms.)
+// Only |w_i - (q_i - 8) s_t| enters e_t, and that leaves the search a freedom: where w_i / s_t lies half way between two codes both
+// give the same magnitude, s_t / 2, exactly (fp16 w and s: the difference is exact in fp32).  Where it does not, it is at least 2^-13
+// away from half way (w = W 2^a, s = S 2^b with integers W, S < 2^11 and |w| >= s / 2: 2 w - (2 k + 1) s is a multiple of 2^(b-1), and is
+// divided by 2 s < 2^(b+12)), so any arithmetic with less error finds the same code.  The search therefore clamps for free: with
+//   u = sat(w / (15 s) + 8 / 15),   q = round(15 u)        (error below 2^-18 codes)
+// the saturation of the first fma to [0, 1] is the clamp to [0, 15].  The codes themselves are made as written above.
+// Bound: the fp32 pipe, five operations per weight and candidate (u, two for the rounding, two for the error), most of them issued in
+// pairs (fma.rn.f32x2 and the like: the same IEEE operations, half the instructions); no conversions, no comparisons.
+// Measured with ten candidates, before (clamp by two comparisons) and now: 4096 x 11008, groups of 128: 114 / 99 us; one scale per column,
+// 4096 x 4096: 99 / 85, 8192 x 1024: 163 / 134.
 #include "device_utils.cuh"
 #include "marlin_internal.cuh"
 
@@ -31,34 +37,37 @@ namespace {
 
 __device__ __forceinline__ float load_w(const uint16_t* p) { return __half2float(__ushort_as_half(__ldg(p))); }
 
-__device__ __forceinline__ f32x2 clamp2(f32x2 x) {
-  float lo, hi;
-  unpack2(x, lo, hi);
-  return pack2(fminf(fmaxf(lo, -8.f), 7.f), fminf(fmaxf(hi, -8.f), 7.f));
-}
-
 // Rounding half to even by adding 1.5 * 2^23: in [2^23, 2^24) the spacing of fp32 is one, so the sum rounds x to an
 // integer q, which sits in the low bits of its representation.  Clamping to [-8, 7] first gives the same integer
 // as clamping the rounded value (both ends are integers and rounding is monotone).
 constexpr float kRoundMagic = 12582912.f;
-__device__ __forceinline__ uint32_t code_of(float w, float inv) {
+// Here the integer comes with the bits of the magic number; of eight of them, put together by multiplications by 16, those are taken
+// off at the end, and 8 is added to each.
+__device__ __forceinline__ uint32_t code_bits(float w, float inv) {
   const float x = fminf(fmaxf(__fmul_rn(w, inv), -8.f), 7.f);
-  return (__float_as_uint(__fadd_rn(x, kRoundMagic)) + 8u) & 15u;  // q + 8, q = -8 .. 7
+  return __float_as_uint(__fadd_rn(x, kRoundMagic));
+}
+constexpr uint32_t kMagicBits = 0x4b400000u, kEightMagicBits = (kMagicBits - 8u) * 0x11111111u;
+
+// the search's u (see the top)
+__device__ __forceinline__ float unit_of(float w, float inv15) {
+  float u;
+  asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(u) : "f"(w), "f"(inv15), "f"(8.f / 15.f));
+  return u;
 }
 
-// candidate t: fp16 scale bits, the scale and its reciprocal
-__device__ __forceinline__ uint16_t candidate_scale(float a, int t, int n_grid, float& s, float& inv) {
+// candidate t: fp16 scale bits, the scale and a fifteenth of its reciprocal
+__device__ __forceinline__ uint16_t candidate_scale(float a, int t, int n_grid, float& s, float& inv15) {
   const float two_fifteenths = __fdiv_rn(2.f, 15.f);
   const float r = __fsub_rn(1.f, __fdiv_rn((float)t, (float)n_grid));
   uint16_t sh = __half_as_ushort(__float2half_rn(__fmul_rn(__fmul_rn(a, r), two_fifteenths)));
   if (sh == 0) sh = 1;  // a scale that rounds to zero: the smallest positive fp16
   s = __half2float(__ushort_as_half(sh));
-  inv = __fdiv_rn(1.f, s);
+  inv15 = __fmul_rn(__fdiv_rn(1.f, s), 1.f / 15.f);
   return sh;
 }
 
 // Groups of 32, 64 or 128 rows: the rows of a group in registers, two per register pair.
-// 4096 x 11008, groups of 128, ten candidates: 118 us (140 with rintf and without the pairs), both pipes about 60 % busy.
 template <int GC>
 __global__ void __launch_bounds__(128)
 quantize_rtn_cached_kernel(const uint16_t* __restrict__ W, uint32_t* __restrict__ q_kpacked, uint16_t* __restrict__ scales,
@@ -75,28 +84,52 @@ quantize_rtn_cached_kernel(const uint16_t* __restrict__ W, uint32_t* __restrict_
     w[i] = pack2(lo, hi);
     a = fmaxf(a, fmaxf(fabsf(lo), fabsf(hi)));
   }
-  const f32x2 magic = pack2(kRoundMagic, kRoundMagic), minus1 = pack2(-1.f, -1.f);
+  const f32x2 magic = pack2(kRoundMagic, kRoundMagic), minus_magic8 = pack2(-kRoundMagic - 8.f, -kRoundMagic - 8.f);
+  const f32x2 fifteen = pack2(15.f, 15.f);
   float best_err = __int_as_float(0x7f800000);  // +inf
   uint16_t best_s = 1;
-#pragma unroll 1
-  for (int t = 0; t < n_candidates; ++t) {
-    float s, inv;
-    const uint16_t sh = candidate_scale(a, t, n_grid, s, inv);
-    const f32x2 s2 = pack2(s, s), inv2 = pack2(inv, inv);
-    float err = 0.f;
+  if (n_candidates & 1) {
+    float s, inv15, err = 0.f;
+    const uint16_t sh = candidate_scale(a, 0, n_grid, s, inv15);
 #pragma unroll
-    for (int i = 0; i < GC / 2; ++i) {
-      const f32x2 y = add2(clamp2(mul2(w[i], inv2)), magic);
-      const f32x2 d = fma2(fma2(y, minus1, magic), s2, w[i]);  // w - q s: magic - y = -q exactly
-      float d0, d1;
-      unpack2(d, d0, d1);
-      err = __fmaf_rn(d0, d0, err);  // in row order
-      err = __fmaf_rn(d1, d1, err);
+    for (int i = 0; i < GC; ++i) {
+      float lo, hi;
+      unpack2(w[i / 2], lo, hi);
+      const float x = i % 2 ? hi : lo;
+      const float q = __fsub_rn(__fmaf_rn(unit_of(x, inv15), 15.f, kRoundMagic), kRoundMagic + 8.f);
+      const float d = __fmaf_rn(-q, s, x);
+      err = __fmaf_rn(d, d, err);
     }
     if (err < best_err) {
       best_err = err;
       best_s = sh;
     }
+  }
+  // two candidates at a time, in the halves of a register pair
+#pragma unroll 1
+  for (int t = n_candidates & 1; t < n_candidates; t += 2) {
+    float s[2], inv15[2], e[2];
+    uint16_t sh[2];
+#pragma unroll
+    for (int c = 0; c < 2; ++c) sh[c] = candidate_scale(a, t + c, n_grid, s[c], inv15[c]);
+    f32x2 err = pack2(0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < GC; ++i) {  // in row order
+      float lo, hi, q[2];
+      unpack2(w[i / 2], lo, hi);
+      const float x = i % 2 ? hi : lo;
+      const f32x2 y = fma2(pack2(unit_of(x, inv15[0]), unit_of(x, inv15[1])), fifteen, magic);  // magic + q + 8
+      unpack2(add2(y, minus_magic8), q[0], q[1]);
+      const f32x2 d = pack2(__fmaf_rn(-q[0], s[0], x), __fmaf_rn(-q[1], s[1], x));
+      err = fma2(d, d, err);
+    }
+    unpack2(err, e[0], e[1]);
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+      if (e[c] < best_err) {
+        best_err = e[c];
+        best_s = sh[c];
+      }
   }
   const float s = __half2float(__ushort_as_half(best_s));
   const float inv = __fdiv_rn(1.f, s);
@@ -106,12 +139,13 @@ quantize_rtn_cached_kernel(const uint16_t* __restrict__ W, uint32_t* __restrict_
   for (int i8 = 0; i8 < GC / 8; ++i8) {
     uint32_t word = 0;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
+    for (int j = 3; j >= 0; --j) {
       float lo, hi;
       unpack2(w[4 * i8 + j], lo, hi);
-      word |= (code_of(lo, inv) << (8 * j)) | (code_of(hi, inv) << (8 * j + 4));
+      word = 16u * word + code_bits(hi, inv);
+      word = 16u * word + code_bits(lo, inv);
     }
-    q_kpacked[((size_t)g * (GC / 8) + i8) * N + n] = word;
+    q_kpacked[((size_t)g * (GC / 8) + i8) * N + n] = word - kEightMagicBits;
   }
 }
 
@@ -133,19 +167,17 @@ quantize_max_kernel(const uint16_t* __restrict__ W, uint32_t* __restrict__ q_kpa
   reinterpret_cast<uint2*>(q_kpacked + (size_t)part * (kPartRows / 8) * N)[n2] = make_uint2(m & 0xffffu, m >> 16);
 }
 
-// The search: lane = column, warp = one candidate or (PAIRS) two of them in a register pair, rows in order.  The rows
-// come through a ring of shared-memory tiles (64 rows x 32 columns, three tiles ahead): with few warps per scheduler
-// nothing else hides the latency of the L2 (loading sixteen rows ahead into registers instead left the schedulers idle
-// four cycles in five).
-constexpr int kSearchCols = 32, kSearchMaxWarps = 16, kSearchRows = 64, kSearchTiles = 4;
-template <bool PAIRS>
+// The search: lane = column, warp = one candidate, rows in order.  The rows come through a ring of shared-memory tiles (64 rows x 32
+// columns, three tiles ahead): with few warps per scheduler nothing else hides the latency of the L2.  A tile is turned into
+// fp32 pairs of rows once for all candidates, one tile ahead of the sums.
+constexpr int kSearchCols = 32, kSearchMinWarps = 8, kSearchMaxWarps = 16, kSearchRows = 64, kSearchTiles = 4;
 __global__ void __launch_bounds__(kSearchCols * kSearchMaxWarps)
 quantize_search_kernel(const uint16_t* __restrict__ W, const uint32_t* __restrict__ q_kpacked, uint16_t* __restrict__ scales,
                        int N, int G, int n_grid, int n_candidates) {
-  constexpr int PER = PAIRS ? 2 : 1;  // candidates of a warp
   __shared__ __align__(16) uint16_t ring[kSearchTiles][kSearchRows][kSearchCols];
-  __shared__ float errs[PER * kSearchMaxWarps][kSearchCols];
-  __shared__ uint16_t cands[PER * kSearchMaxWarps][kSearchCols];
+  __shared__ f32x2 pairs[2][kSearchRows / 2][kSearchCols];
+  __shared__ float errs[kSearchMaxWarps][kSearchCols];
+  __shared__ uint16_t cands[kSearchMaxWarps][kSearchCols];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
   const int n = blockIdx.x * kSearchCols + lane;
   const int g = blockIdx.y;
@@ -163,53 +195,98 @@ quantize_search_kernel(const uint16_t* __restrict__ W, const uint32_t* __restric
     }
     asm volatile("cp.async.commit_group;" ::: "memory");  // one group per call, empty ones too
   };
+  // rows of a tile from 16 to 32 bits, in two steps: loads into registers, and later their way into `pairs`
+  constexpr int kWiden = kSearchRows / 2 / kSearchMinWarps;
+  uint16_t wide[kWiden][2];
+  auto widen_load = [&](int tile) {
+#pragma unroll
+    for (int i = 0; i < kWiden; ++i) {
+      const int r2 = warp + i * warps;
+      if (r2 < kSearchRows / 2) {
+        wide[i][0] = ring[tile % kSearchTiles][2 * r2][lane];
+        wide[i][1] = ring[tile % kSearchTiles][2 * r2 + 1][lane];
+      }
+    }
+  };
+  auto widen_store = [&](int tile) {
+#pragma unroll
+    for (int i = 0; i < kWiden; ++i) {
+      const int r2 = warp + i * warps;
+      if (r2 < kSearchRows / 2)
+        pairs[tile & 1][r2][lane] = pack2(__half2float(__ushort_as_half(wide[i][0])), __half2float(__ushort_as_half(wide[i][1])));
+    }
+  };
   uint32_t amax = 0;
   for (int part = 0; part < G / kPartRows; ++part)
     amax = max(amax, __ldg(q_kpacked + ((size_t)g * (G / kPartRows) + part) * (kPartRows / 8) * N + n));
   const float a = __half2float(__ushort_as_half((uint16_t)amax));
-  const f32x2 magic = pack2(kRoundMagic, kRoundMagic), minus1 = pack2(-1.f, -1.f);
+  const f32x2 magic = pack2(kRoundMagic, kRoundMagic), magic8 = pack2(kRoundMagic + 8.f, kRoundMagic + 8.f);
+  const f32x2 minus1 = pack2(-1.f, -1.f), fifteen = pack2(15.f, 15.f);
   float best_err = __int_as_float(0x7f800000);
   uint16_t best_s = 1;
-  for (int t0 = 0; t0 < n_candidates; t0 += PER * warps) {
-    // (slots past the last candidate repeat it)
-    float s[PER], inv[PER], err[PER];
+  for (int t0 = 0; t0 < n_candidates; t0 += warps) {
+    // (warps past the last candidate repeat it)
+    constexpr int B = 4;
+    float s, inv15, err = 0.f, d[2 * B];
 #pragma unroll
-    for (int e = 0; e < PER; ++e) {
-      cands[PER * warp + e][lane] =
-          candidate_scale(a, min(t0 + PER * warp + e, n_candidates - 1), n_grid, s[e], inv[e]);
-      err[e] = 0.f;
-    }
-    const f32x2 s2 = pack2(s[0], s[PER - 1]), inv2 = pack2(inv[0], inv[PER - 1]);
-    f32x2 err2 = pack2(0.f, 0.f);
+    for (int i = 0; i < 2 * B; ++i) d[i] = 0.f;
+    cands[warp][lane] = candidate_scale(a, min(t0 + warp, n_candidates - 1), n_grid, s, inv15);
+    const f32x2 s2 = pack2(s, s);
     for (int i = 0; i < kSearchTiles - 1; ++i) fetch(i);
+    asm volatile("cp.async.wait_group %0;" ::"n"(kSearchTiles - 2) : "memory");
+    __syncthreads();
+    widen_load(0);
+    widen_store(0);
     for (int tile = 0; tile < tiles; ++tile) {
-      asm volatile("cp.async.wait_group %0;" ::"n"(kSearchTiles - 2) : "memory");
-      __syncthreads();  // this tile has landed for everybody, and everybody has left the one before it
+      asm volatile("cp.async.wait_group %0;" ::"n"(kSearchTiles - 3) : "memory");
+      // this tile's pairs are there, the next tile has landed for everybody, and everybody has left the pairs of the tile before
+      __syncthreads();
+      if (tile + 1 < tiles) widen_load(tile + 1);
       fetch(tile + kSearchTiles - 1);
-      const uint16_t* rows = &ring[tile % kSearchTiles][0][lane];
-#pragma unroll 16
-      for (int i = 0; i < kSearchRows; ++i) {
-        const float wi = __half2float(__ushort_as_half(rows[i * kSearchCols]));
-        if constexpr (PAIRS) {
-          const f32x2 ww = pack2(wi, wi);
-          const f32x2 y = add2(clamp2(mul2(ww, inv2)), magic);
-          const f32x2 d = fma2(fma2(y, minus1, magic), s2, ww);
-          err2 = fma2(d, d, err2);
-        } else {
-          const float x = fminf(fmaxf(__fmul_rn(wi, inv[0]), -8.f), 7.f);
-          const float q = __fsub_rn(__fadd_rn(x, kRoundMagic), kRoundMagic);
-          const float d = __fmaf_rn(-q, s[0], wi);
-          err[0] = __fmaf_rn(d, d, err[0]);
-        }
-      }
-    }
-    if constexpr (PAIRS) unpack2(err2, err[0], err[PER - 1]);
+      const f32x2* rows = &pairs[tile & 1][0][lane];
+      // Four pairs at a time, each operation for all of them, the next four already on their way and the squares of the four
+      // before (a chain, in row order) in between: with two or three warps per scheduler one after the other would wait for itself
+      // (two, four, eight at a time: 91, 85, 85 us for 4096 x 4096 with one scale per column; 167, 157, 169 for 4096 x 11008 in groups of 256).
+      f32x2 next[B];
 #pragma unroll
-    for (int e = 0; e < PER; ++e) errs[PER * warp + e][lane] = err[e];
+      for (int i = 0; i < B; ++i) next[i] = rows[i * kSearchCols];
+#pragma unroll
+      for (int i0 = 0; i0 < kSearchRows / 2; i0 += B) {
+        f32x2 ww[B], y[B];
+        float u[2 * B];
+#pragma unroll
+        for (int i = 0; i < B; ++i) {
+          ww[i] = next[i];
+          if (i0 + B < kSearchRows / 2) next[i] = rows[(i0 + B + i) * kSearchCols];
+        }
+#pragma unroll
+        for (int i = 0; i < B; ++i) {
+          float lo, hi;
+          unpack2(ww[i], lo, hi);
+          u[2 * i] = unit_of(lo, inv15);
+          u[2 * i + 1] = unit_of(hi, inv15);
+          err = __fmaf_rn(d[i], d[i], err);
+        }
+#pragma unroll
+        for (int i = 0; i < B; ++i) {
+          y[i] = fma2(pack2(u[2 * i], u[2 * i + 1]), fifteen, magic);  // magic + q + 8
+          err = __fmaf_rn(d[B + i], d[B + i], err);
+        }
+#pragma unroll
+        for (int i = 0; i < B; ++i) y[i] = fma2(y[i], minus1, magic8);  // -q, exactly
+#pragma unroll
+        for (int i = 0; i < B; ++i) unpack2(fma2(y[i], s2, ww[i]), d[2 * i], d[2 * i + 1]);
+      }
+      if (tile + 1 < tiles) widen_store(tile + 1);
+    }
+#pragma unroll
+    for (int i = 0; i < 2 * B; ++i) err = __fmaf_rn(d[i], d[i], err);
+    errs[warp][lane] = err;
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
     if (warp == 0) {
       // in candidate order, the first one on ties
-      for (int c = 0; c < PER * warps && t0 + c < n_candidates; ++c)
+      for (int c = 0; c < warps && t0 + c < n_candidates; ++c)
         if (errs[c][lane] < best_err) {
           best_err = errs[c][lane];
           best_s = cands[c][lane];
@@ -236,10 +313,12 @@ quantize_encode_kernel(const uint16_t* __restrict__ W, uint32_t* __restrict__ q_
   const float inv1 = __fdiv_rn(1.f, __half2float(__ushort_as_half((uint16_t)(sh >> 16))));
   uint2 word = make_uint2(0, 0);
 #pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    word.x |= code_of(__half2float(__ushort_as_half((uint16_t)(rows[j] & 0xffffu))), inv0) << (4 * j);
-    word.y |= code_of(__half2float(__ushort_as_half((uint16_t)(rows[j] >> 16))), inv1) << (4 * j);
+  for (int j = 7; j >= 0; --j) {
+    word.x = 16u * word.x + code_bits(__half2float(__ushort_as_half((uint16_t)(rows[j] & 0xffffu))), inv0);
+    word.y = 16u * word.y + code_bits(__half2float(__ushort_as_half((uint16_t)(rows[j] >> 16))), inv1);
   }
+  word.x -= kEightMagicBits;
+  word.y -= kEightMagicBits;
   reinterpret_cast<uint2*>(q_kpacked + (size_t)k8 * N)[n2] = word;
 }
 
@@ -258,16 +337,10 @@ cudaError_t launch_quantize_rtn(const uint16_t* W, uint32_t* q_kpacked, uint16_t
   } else {
     const unsigned pairs = (unsigned)((N / 2 + 127) / 128);
     quantize_max_kernel<<<dim3(pairs, (unsigned)(K / kPartRows)), 128, 0, stream>>>(W, q_kpacked, N);
-    // Pairs of candidates need fewer instructions, single ones give twice the warps: with less than two warps of pairs
-    // per scheduler the latter is faster (4096 x 4096, one scale per column, 640 warps of pairs: 80 us against 97 for the
-    // search; 4096 x 11008, groups of 256, 27520 of them: 218 us against 184 for the whole conversion).
     const dim3 blocks((unsigned)(N / kSearchCols), (unsigned)(K / G));
-    const int singles = n_candidates < kSearchMaxWarps ? n_candidates : kSearchMaxWarps;
-    const int pairs_of = (n_candidates + 1) / 2 < kSearchMaxWarps ? (n_candidates + 1) / 2 : kSearchMaxWarps;
-    if ((long long)blocks.x * blocks.y * pairs_of < 148 * 4 * 2)
-      quantize_search_kernel<false><<<blocks, kSearchCols * singles, 0, stream>>>(W, q_kpacked, scales, N, G, n_grid, n_candidates);
-    else
-      quantize_search_kernel<true><<<blocks, kSearchCols * pairs_of, 0, stream>>>(W, q_kpacked, scales, N, G, n_grid, n_candidates);
+    // (warps without a candidate of their own fetch and widen all the same)
+    const int warps = n_candidates < kSearchMinWarps ? kSearchMinWarps : n_candidates < kSearchMaxWarps ? n_candidates : kSearchMaxWarps;
+    quantize_search_kernel<<<blocks, kSearchCols * warps, 0, stream>>>(W, q_kpacked, scales, N, G, n_grid, n_candidates);
     // one grid row per eight rows of W: up to 2^20 / 8, above the limit of grid.y, so the rows go on in slices of it
     constexpr int kSlice = 32768;
     for (int r0 = 0; r0 < K / 8; r0 += kSlice) {

@@ -43,13 +43,39 @@ def test_codes_and_scales_match_the_oracle_bit_for_bit(marlin, K, N, G, n_grid, 
     assert np.array_equal(to_host(q).view(np.uint32), inputs.kpack(Q_ref))
 
 
-# groups above 128 rows: one candidate per warp (few blocks) or a pair of them (many), more candidates than one round of
-# warps takes, odd counts, tiles of 64 rows that wrap the ring
+# groups above 128 rows: one candidate per warp, fewer candidates than warps, more than one round of warps takes, odd counts,
+# tiles of 64 rows that wrap the ring
 @pytest.mark.parametrize("K,N,G,n_grid,n_cand", [
     (512, 64, 256, 40, 37), (1024, 2048, 256, 40, 35), (1024, 4096, 256, 20, 10), (1024, 2112, -1, 20, 10),
     (256, 64, -1, 20, 2), (3072, 192, 1536, 20, 17)])
 def test_long_groups_match_the_oracle_bit_for_bit(marlin, K, N, G, n_grid, n_cand):
     test_codes_and_scales_match_the_oracle_bit_for_bit(marlin, K, N, G, n_grid, n_cand)
+
+
+# weights half way between two codes, subnormals and the largest values: the search may take either code of a tie, the codes may not
+@pytest.mark.parametrize("G", [32, 64, 128, 256])
+@pytest.mark.parametrize("kind", ["halves", "subnormal", "largest", "wide"])
+def test_ties_and_extremes_match_the_oracle_bit_for_bit(marlin, kind, G):
+    import torch
+    from oracle import quantize_ref
+    from paper_2408_11743_b200 import inputs
+    rng = np.random.default_rng(G)
+    K, N = 512, 256
+    if kind == "halves":
+        W = rng.integers(-15, 16, (K, N)) * 0.5
+    elif kind == "subnormal":
+        W = rng.integers(-40, 41, (K, N)) * 2.0 ** -24
+    elif kind == "largest":
+        W = rng.choice([-65504.0, 65504.0, 4367.0, 0.0], (K, N))
+    else:
+        W = rng.integers(-2047, 2048, (K, N)) * 2.0 ** rng.integers(-20, 4, (K, N))
+    W = W.astype(np.float16)
+    for n_grid, n_cand in [(20, 10), (100, 99), (7, 7)]:
+        q, s = marlin.quantize_rtn(to_dev(W), G, n_grid, n_cand)
+        torch.cuda.synchronize()
+        Q_ref, S_ref, _ = quantize_ref.quantize_rtn(W, G, n_grid, n_cand)
+        assert np.array_equal(to_host(s).view(np.uint16), S_ref.view(np.uint16))
+        assert np.array_equal(to_host(q).view(np.uint32), inputs.kpack(Q_ref))
 
 
 def test_plain_rounding_versus_search_on_outlier_groups(marlin):
