@@ -42,8 +42,8 @@
 //
 // Partition: every column tile is cut into S k-ranges, one per CTA, where that keeps most SMs busy (one
 // epilogue per CTA, all CTAs alike); else even stripes over all units.  Fix-up of a shared tile: the CTAs of a
-// tile form thread-block clusters; every CTA leaves its partial tile in a workspace slot, and behind one cluster barrier
-// every CTA adds up its share of the tile.  What several clusters (or stripes) hold of a tile goes through further slots,
+// tile form thread-block clusters; every CTA leaves what belongs to the others in a workspace slot, and behind one cluster barrier
+// adds the others' parts to its own share of the tile.  What several clusters (or stripes) hold of a tile goes through further slots,
 // and the last arriver adds them in worker order.  The order of the fp32 sum is always the same: the same inputs give
 // the same bits.  Bounded waits and programmatic dependent launch are those of the small-batch kernel (gemm_dense.cu).
 #pragma once
@@ -317,42 +317,44 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
   // first and last tile)
   auto slot_ptr = [&](uint32_t index) { return reinterpret_cast<float4*>(p.partials + (size_t)index * (G::TN * MPAD)); };
   // Blocks x of a tile (x = c32 * nb + b, every `step`-th from x0 on) summed over the slots slot(0) .. slot(n - 1), in order;
-  // done(c32, b, f) takes the sums.  Two blocks and two slots at a time: eight 16-byte loads of a lane are in flight together.  What a slot
+  // done(c32, b, f) takes the sums.  Two blocks and two slots at a time, or one block and four slots where that is all a warp
+  // has (deferred scales, 32 rows: 20 x 11008 x 1088 8.4 us, 7.8 so): eight 16-byte loads of a lane are in flight together.  What a slot
   // held is cleared behind its last read, so that a workspace comes back from most calls as it was given (not with deferred scales, and
   // not past the last column); nothing relies on it: slots are written before they are read.
-  auto sum_blocks = [&](int x0, int step, int items, int nb, uint32_t col, int n, auto slot, auto done) {
-    for (int x = x0; x < items; x += 2 * step) {
-      int c32[2], b[2];
-      bool ok[2];
+  auto sum_some = [&](auto ib_c, int x0, int step, int items, int nb, uint32_t col, int n, auto slot, auto done) {
+    constexpr int IB = decltype(ib_c)::value, QN = 4 / IB;
+    for (int x = x0; x < items; x += IB * step) {
+      int c32[IB], b[IB];
+      bool ok[IB];
 #pragma unroll
-      for (int i = 0; i < 2; ++i) {
+      for (int i = 0; i < IB; ++i) {
         const int xi = x + i * step;
         c32[i] = xi / nb;
         b[i] = xi - c32[i] * nb;
         ok[i] = xi < items && col * G::TN + (uint32_t)c32[i] * 32 < (uint32_t)p.N;
       }
-      float f[2][8];
+      float f[IB][8];
 #pragma unroll
-      for (int i = 0; i < 2; ++i)
+      for (int i = 0; i < IB; ++i)
 #pragma unroll
         for (int e = 0; e < 8; ++e) f[i][e] = 0.f;
-      for (int src = 0; src < n; src += 2) {
-        float4 v[2][2][2];
+      for (int src = 0; src < n; src += QN) {
+        float4 v[QN][IB][2];
 #pragma unroll
-        for (int q = 0; q < 2; ++q)
+        for (int q = 0; q < QN; ++q)
           if (src + q < n) {
             const float4* from = slot(src + q);
 #pragma unroll
-            for (int i = 0; i < 2; ++i)
+            for (int i = 0; i < IB; ++i)
 #pragma unroll
               for (int h = 0; h < 2; ++h)
                 if (ok[i]) v[q][i][h] = ld_cg_f4(from + frag_index(c32[i], b[i], h));
           }
 #pragma unroll
-        for (int q = 0; q < 2; ++q)
+        for (int q = 0; q < QN; ++q)
           if (src + q < n) {
 #pragma unroll
-            for (int i = 0; i < 2; ++i)
+            for (int i = 0; i < IB; ++i)
 #pragma unroll
               for (int h = 0; h < 2; ++h) {
                 f[i][4 * h] += v[q][i][h].x; f[i][4 * h + 1] += v[q][i][h].y;
@@ -361,11 +363,11 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
           }
         if constexpr (!DEF) {
 #pragma unroll
-          for (int q = 0; q < 2; ++q)
+          for (int q = 0; q < QN; ++q)
             if (src + q < n) {
               float4* to = slot(src + q);
 #pragma unroll
-              for (int i = 0; i < 2; ++i)
+              for (int i = 0; i < IB; ++i)
 #pragma unroll
                 for (int h = 0; h < 2; ++h)
                   if (ok[i]) to[frag_index(c32[i], b[i], h)] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -373,9 +375,15 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
         }
       }
 #pragma unroll
-      for (int i = 0; i < 2; ++i)
+      for (int i = 0; i < IB; ++i)
         if (ok[i]) done(c32[i], b[i], f[i], i);
     }
+  };
+  auto sum_blocks = [&](int x0, int step, int items, int nb, uint32_t col, int n, auto slot, auto done) {
+    if (DEF && MPAD == 32 && x0 + step >= items)
+      sum_some(IntC<1>{}, x0, step, items, nb, col, n, slot, done);
+    else
+      sum_some(IntC<2>{}, x0, step, items, nb, col, n, slot, done);
   };
   // sums to C
   auto store_block = [&](int c32, int b, const float (&f)[8], int i, uint32_t col, int m_lim, size_t row0) {
@@ -530,19 +538,20 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
         store_block(c32, c / NT * 2 + b, fb, b, col, m_lim, row0);
       }
     };
-    // Piece c of n partial tiles in their order: tile `own` (n: none) from tensor memory, the others from their slots, two of them on
-    // their way at a time, and cleared behind the read (a workspace comes back as it was given).
+    // Piece c of n partial tiles in their order: tile `own` (n: none) from tensor memory, the others from their slots, three of them
+    // on their way at a time (a cluster of four: one latency of the L2), and cleared behind the read (a workspace comes back as it was given).
     auto gather = [&](int c, int n, int own, auto slot, float (&sum)[16]) {
       float f[16];
       if (own < n) own_sums(c, f);
 #pragma unroll
       for (int x = 0; x < 16; ++x) sum[x] = 0.f;
       const int others = own < n ? n - 1 : n;
-      for (int o = 0; o < others; o += 2) {
-        float4 v[2][4];
-        float4* from[2];
+      constexpr int UN = 3;
+      for (int o = 0; o < others; o += UN) {
+        float4 v[UN][4];
+        float4* from[UN];
 #pragma unroll
-        for (int i = 0; i < 2; ++i)
+        for (int i = 0; i < UN; ++i)
           if (o + i < others) {
             from[i] = slot(o + i + (o + i >= own ? 1 : 0));
 #pragma unroll
@@ -550,7 +559,7 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
               if (in_rows(c, y)) v[i][y] = ld_cg_f4(from[i] + piece_index(c, y));
           }
 #pragma unroll
-        for (int i = 0; i < 2; ++i)
+        for (int i = 0; i < UN; ++i)
           if (o + i < others) {
             if (o + i == own) {
 #pragma unroll
