@@ -357,8 +357,8 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
             for (int i = 0; i < IB; ++i)
 #pragma unroll
               for (int h = 0; h < 2; ++h) {
-                f[i][4 * h] += v[q][i][h].x; f[i][4 * h + 1] += v[q][i][h].y;
-                f[i][4 * h + 2] += v[q][i][h].z; f[i][4 * h + 3] += v[q][i][h].w;
+                f[i][4 * h] = __fadd_rn(f[i][4 * h], v[q][i][h].x); f[i][4 * h + 1] = __fadd_rn(f[i][4 * h + 1], v[q][i][h].y);
+                f[i][4 * h + 2] = __fadd_rn(f[i][4 * h + 2], v[q][i][h].z); f[i][4 * h + 3] = __fadd_rn(f[i][4 * h + 3], v[q][i][h].w);
               }
           }
         if constexpr (!DEF) {
@@ -479,7 +479,9 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
       sc[0] = s01.x; sc[1] = s01.y; sc[2] = s23.x; sc[3] = s23.y;
     }
   };
-  // 16 rows from row m on out of tensor memory, the halves of the k-blocks added, scaled: f[8b + 4h + e]
+  // 16 rows from row m on out of tensor memory, the halves of the k-blocks added, scaled: f[8b + 4h + e].  Every product and sum of the
+  // fix-up is rounded by itself (no fma): whether a CTA's part goes into the sum from registers or through a slot depends on who
+  // comes first and must not show.
   auto load_rows = [&](int t, int m, const float (&sc)[4], float (&f)[16]) {
     float a[2][8], a2[2][8];
 #pragma unroll
@@ -493,8 +495,8 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
     for (int x = 0; x < 16; ++x) {
       const int h = (x >> 2) & 1, i = 4 * (x >> 3) + (x & 3);
       f[x] = a[h][i];
-      if constexpr (KH == 2) f[x] += a2[h][i];
-      if constexpr (SCALE == kPerColumn) f[x] *= sc[2 * h + ((x >> 1) & 1)];
+      if constexpr (KH == 2) f[x] = __fadd_rn(f[x], a2[h][i]);
+      if constexpr (SCALE == kPerColumn) f[x] = __fmul_rn(f[x], sc[2 * h + ((x >> 1) & 1)]);
     }
   };
   // The CTA's last tile (not with deferred scales): the converters have nothing else left to do, so all 16 warps read it out, in pieces
@@ -563,19 +565,20 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
           if (o + i < others) {
             if (o + i == own) {
 #pragma unroll
-              for (int x = 0; x < 16; ++x) sum[x] += f[x];
+              for (int x = 0; x < 16; ++x) sum[x] = __fadd_rn(sum[x], f[x]);
             }
 #pragma unroll
             for (int y = 0; y < 4; ++y)
               if (in_rows(c, y)) {
-                sum[4 * y] += v[i][y].x; sum[4 * y + 1] += v[i][y].y; sum[4 * y + 2] += v[i][y].z; sum[4 * y + 3] += v[i][y].w;
+                sum[4 * y] = __fadd_rn(sum[4 * y], v[i][y].x); sum[4 * y + 1] = __fadd_rn(sum[4 * y + 1], v[i][y].y);
+                sum[4 * y + 2] = __fadd_rn(sum[4 * y + 2], v[i][y].z); sum[4 * y + 3] = __fadd_rn(sum[4 * y + 3], v[i][y].w);
                 from[i][piece_index(c, y)] = make_float4(0.f, 0.f, 0.f, 0.f);
               }
           }
       }
       if (own == n - 1) {
 #pragma unroll
-        for (int x = 0; x < 16; ++x) sum[x] += f[x];
+        for (int x = 0; x < 16; ++x) sum[x] = __fadd_rn(sum[x], f[x]);
       }
     };
     pdl_wait_prior_grids();

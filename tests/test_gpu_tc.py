@@ -138,3 +138,48 @@ def test_fused_activation_on_the_way_out(marlin, M, I, G):
     err = np.abs(to_host(H).astype(np.float64) - want)
     assert np.all(err <= 2.0 ** -10.9 * np.abs(want) + 2.0 ** -25 + 1e-9)
     assert bool(big[:guard].isnan().all()) and bool(big[guard + M * I:].isnan().all())
+
+
+# One scale per column: every CTA scales its exact integer sums, each product rounded to fp32, and the parts are added in worker order, each
+# sum rounded; a product that entered a sum unrounded would show in about one result of 2^13.  k-ranges without clusters and stripes
+# (a CTA adds onto its own part or goes through a slot, by who comes last), one cluster per tile, two.
+@pytest.mark.parametrize("tile", ["128", "256"])
+@pytest.mark.parametrize("split,cluster", [(3, 0), (0, 0), (3, 3), (4, 4), (4, 2)])
+def test_scaled_parts_are_rounded_and_added_in_worker_order(marlin, monkeypatch, tile, split, cluster):
+    import torch
+    for k, v in (("TILE", tile), ("SPLIT", split), ("CLUSTER", cluster)):
+        monkeypatch.setenv("MARLIN_B200_TC_" + k, str(v))
+    M, K, N = 128, 3072, 4096
+    rng = np.random.default_rng(split + cluster)
+    Q = rng.integers(0, 16, size=(K, N), dtype=np.uint8)
+    A = to_dev(rng.integers(-3, 4, size=(M, K)).astype(np.float16))
+    S = (rng.random((1, N)) * 0.015 + 0.005).astype(np.float16)
+    layer = DenseLayer(marlin, inputs.kpack(Q), S, -1, max_M=M)
+    W, s = to_dev(Q).double() - 8, to_dev(S).float()
+    KB, TN = K // 128, int(tile)
+    tiles = N // TN
+    workers = split * tiles if split else min(KB * tiles, torch.cuda.get_device_properties(0).multi_processor_count)
+    cuts = {t * KB + r * KB // split for t in range(tiles) for r in range(split)} if split else {w * KB * tiles // workers for w in range(workers)}
+    want = torch.empty(M, N, dtype=torch.float16, device="cuda")
+    for t in range(tiles):
+        col = slice(t * TN, (t + 1) * TN)
+        edges = sorted({t * KB, (t + 1) * KB} | {c for c in cuts if t * KB < c < (t + 1) * KB})
+        parts = []
+        for u0, u1 in zip(edges, edges[1:]):
+            k = slice((u0 - t * KB) * 128, (u1 - t * KB) * 128)
+            parts.append((A[:, k].double() @ W[k, col]).float() * s[:, col])
+        per = cluster if cluster > 1 else len(parts)
+        shares = []
+        for c in range(0, len(parts), per):
+            shares.append(parts[c])
+            for part in parts[c + 1:c + per]:
+                shares[-1] = shares[-1] + part
+        total = shares[0]
+        for share in shares[1:]:
+            total = total + share
+        want[:, col] = total.half()
+    for _ in range(20):
+        C = marlin.gemm(A, layer.w, layer.s, K, N, K, layer.ws)
+        torch.cuda.synchronize()
+        assert marlin.read_status(layer.ws) == 0
+        assert torch.equal(C, want), int((C != want).sum())
