@@ -29,7 +29,6 @@ cudaError_t launch_gemm_tc(GemmParams p, int sm_count, bool sparse24, bool w8, c
   // paragraph): one launch, its stripes running over (column tile, slab, k-block)
   p.slabs = (uint32_t)((p.M + mpad - 1) / mpad);
   const int format = w8 ? kTcDense8 : sparse24 ? kTcSparse4 : scale == tc::kDeferred ? kTcDeferred4 : p.zq ? kTcZero4 : kTcDense4;
-  p.slab_rows = (uint32_t)tc_slab_rows(format, p.M);
   const TcPlan best = plan_tc(format, p.M, (int)p.kb, p.N, sm_count, kMaxWorkers);
   p.ncols = (int)best.ncols;
   p.units = (uint32_t)(best.ncols * (long long)p.kb);
@@ -38,6 +37,7 @@ cudaError_t launch_gemm_tc(GemmParams p, int sm_count, bool sparse24, bool w8, c
   p.cluster = (uint32_t)best.cluster;
   p.whole = best.whole ? 1u : 0u;
   const int nt = best.nt;
+  p.slab_rows = (uint32_t)tc_slab_rows(format, p.M, nt);
   if (w8) return tc::launch_w8(nt, mpad, scale, p, stream);
   if (sparse24) return tc::launch_sparse(nt, mpad, scale, p, stream);
   return tc::launch_dense(nt, mpad, scale, p, stream);

@@ -51,6 +51,7 @@
 
 #include "device_utils.cuh"
 #include "marlin_internal.cuh"
+#include "tc_plan.h"
 #include "tc_utils.cuh"
 
 namespace marlin_b200 {
@@ -123,6 +124,7 @@ struct Geometry {
   static constexpr int SLOTS = imin(imin((kTmemCols - D_COLS) / SLOT_COLS, kMaxSlots), A_STAGES);
   static constexpr int A_COL0 = kTmemCols - SLOTS * SLOT_COLS;
   static constexpr int RB = MPAD / 8;                      // blocks of eight batch rows
+  static constexpr bool FIXED_ROWS = tc_fixed_rows(DEF, MPAD, NT);  // slabs of MPAD rows, always
   static_assert(W_STAGES >= 3 && A_STAGES >= 3 && SLOTS >= 2 && SLOTS <= A_STAGES, "pipeline");
   static_assert(A_STAGES <= kMaxAStages && W_STAGES <= kMaxWStages, "barrier area");
   static_assert(A_COL0 >= D_COLS && A_COL0 % 2 == 0 && SLOT_COLS % 2 == 0, "tensor memory");
@@ -194,6 +196,9 @@ template <int V>
 struct IntC {
   static constexpr int value = V;
 };
+struct Int {
+  int value;
+};
 
 // ---- the kernel ---------------------------------------------------------------------------------------------------
 template <int NT, int MPAD, int SCALE, int FMT>
@@ -234,8 +239,8 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
                       : p.whole ? stripe_begin32(worker + 1, (uint32_t)p.ncols, P) * KB
                                 : stripe_begin32(worker + 1, U, P);
   const uint32_t total = u1 - u0;  // k-blocks of this CTA
-  // Rows of a slab: a multiple of 16, at most MPAD.  (Deferred scales: always MPAD, see tc_slab_rows.)
-  const uint32_t slab_rows = DEF ? (uint32_t)MPAD : p.slab_rows;
+  // rows of a slab: a multiple of 16, at most MPAD (see tc_slab_rows)
+  const uint32_t slab_rows = G::FIXED_ROWS ? (uint32_t)MPAD : p.slab_rows;
   const bool zp = SCALE != kPerColumn && p.zq != nullptr;  // zero points: rows of the same shape and order as the scales
 
   pdl_launch_dependents();
@@ -720,14 +725,14 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
       }
     } else if (elect_one()) {
       // ------------------------------- MMA issuers (one thread each) -------------------------------------------------
-      // N: the rows of a slab; the halves of an activation tile lie that many rows apart
-      const uint32_t idesc = instr_desc_f16(128, (int)slab_rows), half_step = slab_rows * 8u;
       constexpr int KS = 8 / KH;  // K = 16 steps per warp and k-block
       const int mw = warp - kMmaWarp0;
       const int t = NT == 2 ? mw : 0;
       const int h = KH == 2 ? mw : 0;  // half of the k-block
-      // the MMAs of the k-block in stage s and operand slot `slot` into d_tmem; `fresh`: overwrite what is there
-      auto issue = [&](uint32_t s, uint32_t slot, uint32_t d_tmem, bool fresh) {
+      // the MMAs of the k-block in stage s and operand slot `slot` into d_tmem; `fresh`: overwrite what is there.  N: the rows of
+      // a slab (`rows.value`); the halves of an activation tile lie that many rows apart.
+      auto issue = [&](auto rows, uint32_t s, uint32_t slot, uint32_t d_tmem, bool fresh) {
+        const uint32_t idesc = instr_desc_f16(128, (int)rows.value), half_step = (uint32_t)rows.value * 8u;
         // descriptor of the first K = 16 step of the stage; the others differ in the address field only
         const uint64_t desc0 = smem_desc_k_sw128(smem_u32(a_ring) + s * (uint32_t)G::A_BYTES);
         const uint32_t slot_col = tmem_base + (uint32_t)G::A_COL0 + slot * (uint32_t)G::SLOT_COLS;
@@ -766,7 +771,7 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
               mbar_wait(&dempty[d], d_par, abort_flag, p.status);
             }
             tc_fence_after_sync();
-            issue(s, slot, tmem_base + d * (uint32_t)MPAD, true);
+            issue(IntC<MPAD>{}, s, slot, tmem_base + d * (uint32_t)MPAD, true);
             const uint32_t d_now = d, s_now = s;
             if (++s == (uint32_t)AS) {
               s = 0;
@@ -793,28 +798,43 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
           mbar_wait(&xfull[s], (it / AS) & 1u, abort_flag, p.status);
           mbar_wait(&afull[slot], (it / NSLOTS) & 1u, abort_flag, p.status);
           tc_fence_after_sync();
-          issue((uint32_t)s, (uint32_t)slot, tmem_base + (uint32_t)(d * MPAD), true);
+          issue(IntC<MPAD>{}, (uint32_t)s, (uint32_t)slot, tmem_base + (uint32_t)(d * MPAD), true);
           tc_commit(&dfull[d]);
           tc_commit(&mdone[s]);
         }
       } else {
         const uint32_t d_tmem = tmem_base + (uint32_t)((t * KH + h) * MPAD);
-        uint32_t it = 0, seg = 0;
-        for (uint32_t u = u0; u < u1; ++seg) {
-          const uint32_t len = min(KB - u % KB, u1 - u);
-          // the accumulators are overwritten by the first MMA of the segment: the previous one must be read out
-          if (seg > 0) mbar_wait(&dempty[t], (seg - 1) & 1u, abort_flag, p.status);
-          for (uint32_t x = 0; x < len; ++x, ++it) {
-            const int s = (int)(it % AS), slot = (int)(it % NSLOTS);
-            mbar_wait(&xfull[s], (it / AS) & 1u, abort_flag, p.status);
-            mbar_wait(&afull[slot], (it / NSLOTS) & 1u, abort_flag, p.status);
-            tc_fence_after_sync();
-            issue((uint32_t)s, (uint32_t)slot, d_tmem, x == 0);
-            // one arrival when these MMAs are done: the slot may be rewritten, the activation tile refilled
-            tc_commit(&mdone[s]);
-            if (x + 1 == len) tc_commit(&dfull[t]);
+        auto run = [&](auto rows) {
+          uint32_t it = 0, seg = 0;
+          for (uint32_t u = u0; u < u1; ++seg) {
+            const uint32_t len = min(KB - u % KB, u1 - u);
+            // the accumulators are overwritten by the first MMA of the segment: the previous one must be read out
+            if (seg > 0) mbar_wait(&dempty[t], (seg - 1) & 1u, abort_flag, p.status);
+            for (uint32_t x = 0; x < len; ++x, ++it) {
+              const int s = (int)(it % AS), slot = (int)(it % NSLOTS);
+              mbar_wait(&xfull[s], (it / AS) & 1u, abort_flag, p.status);
+              mbar_wait(&afull[slot], (it / NSLOTS) & 1u, abort_flag, p.status);
+              tc_fence_after_sync();
+              issue(rows, (uint32_t)s, (uint32_t)slot, d_tmem, x == 0);
+              // one arrival when these MMAs are done: the slot may be rewritten, the activation tile refilled
+              tc_commit(&mdone[s]);
+              if (x + 1 == len) tc_commit(&dfull[t]);
+            }
+            u += len;
           }
-          u += len;
+        };
+        // The rows as a constant where there are one or two of them: from a register they take the issuer, which is on the critical path
+        // of a short launch, 1 to 4 % longer (4096 x 4096 at 64 rows 8.87 us so, 8.70 with the constant; a loop for each of 48 and 64 rows
+        // costs as much again, 8.03 / 7.84 behind the other changes of that instance).  At 128 rows, where there are four, it does not show.
+        if constexpr (G::FIXED_ROWS) {
+          run(IntC<MPAD>{});
+        } else if constexpr (MPAD == 32) {
+          if (slab_rows == 16)
+            run(IntC<16>{});
+          else
+            run(IntC<32>{});
+        } else {
+          run(Int{(int)slab_rows});
         }
       }
     }

@@ -8,16 +8,20 @@ namespace marlin_b200 {
 // how the weights reach the MMAs, as far as the cost of a k-block goes
 enum TcFormat { kTcDense4 = 0, kTcSparse4 = 1, kTcDense8 = 2, kTcDeferred4 = 3, kTcZero4 = 4 };
 
-// rows of a slab: the MMA's N
+// the kernel's instance: the most rows that a slab of it has
 inline int tc_mpad(int m) { return m <= 32 ? 32 : (m <= 64 ? 64 : 128); }
 
-// Batches are cut into equal slabs, in units of 16 rows: what MMAs, copies and read-out cost goes with the rows of a slab, so 130 rows are two
-// slabs of 80, not of 128 (8192 x 8192 at 130 rows 25.1 us so, 24.1 now; 4096 x 22016 at 100 rows 25.6 / 24.6; 2:4, 4096 x 4096 at 300 rows
-// 12.6 / 12.2).  With deferred scales the round trip of the accumulators bounds the loop, and an issuer that reads the rows at run time
-// makes it longer: those slabs are whole (128 rows of 4096 x 5504 12.2 us, 12.6 with the same rows at run time).
-inline int tc_slab_rows(int format, int m) {
+// Rows of a slab, the MMA's N.  From 65 rows on a batch is cut into equal slabs, in units of 16 rows: what MMAs and copies cost goes with the
+// rows of a slab, so 130 rows are two slabs of 80, not of 128 (8192 x 8192 at 130 rows 25.1 us so, 24.1 now; 4096 x 22016 at 100 rows
+// 25.6 / 24.6; 2:4, 4096 x 4096 at 300 rows 12.6 / 12.2).  Up to 16 rows on tiles of 256 columns a slab has 16 (28672 x 8192 with one scale per
+// column 25.6 us with 32, 25.3 so; 2:4, 8192 x 8192 at four rows 10.3 / 9.7).  The others are as high as the instance: rows that the issuer has
+// to read at run time, or two loops for two heights, cost what the smaller MMAs give or more (4096 x 4096 at 24 rows 7.44 us with loops for 16 and
+// 32 rows, 7.22 with one; at 48 rows 7.64 and no change).  With deferred scales the round trip of the accumulators bounds the loop, and
+// rows at run time make it longer at every height (128 rows of 4096 x 5504 12.2 us, 12.6 with the same rows at run time).
+constexpr bool tc_fixed_rows(bool deferred, int mpad, int nt) { return deferred || mpad == 64 || (mpad == 32 && nt == 1); }
+inline int tc_slab_rows(int format, int m, int nt) {
   const int mpad = tc_mpad(m), slabs = (m + mpad - 1) / mpad;
-  return format == kTcDeferred4 ? mpad : ((m + slabs - 1) / slabs + 15) / 16 * 16;
+  return tc_fixed_rows(format == kTcDeferred4, mpad, nt) ? mpad : ((m + slabs - 1) / slabs + 15) / 16 * 16;
 }
 
 struct TcPlan {
@@ -116,7 +120,7 @@ inline TcPlan plan_tc_tile(int nt, int format, int rows, int slabs, int kb, int 
 // M rows on a layer of N columns and kb k-blocks; deferred scales have tiles of 128 columns alone
 inline TcPlan plan_tc(int format, int M, int kb, int N, int sm_count, int max_workers) {
   const int mpad = tc_mpad(M), slabs = (M + mpad - 1) / mpad;
-  const int rows = slabs == 1 ? M : tc_slab_rows(format, M);
+  const int rows = slabs == 1 ? M : tc_slab_rows(format, M, 1);  // (several slabs: the same with both tile widths)
   const char* columns = getenv("MARLIN_B200_TC_TILE");  // tuning knob: 128 or 256 columns per tile, where there is a choice
   TcPlan best{};
   for (int nt = 1; nt <= 2; ++nt) {

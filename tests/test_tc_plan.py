@@ -17,21 +17,25 @@ extern "C" void plan(int format, int M, int kb, int N, int sms, int most, long l
   const marlin_b200::TcPlan p = marlin_b200::plan_tc(format, M, kb, N, sms, most);
   out[0] = p.nt; out[1] = p.whole; out[2] = p.split; out[3] = p.cluster; out[4] = p.workers; out[5] = p.ncols;
 }
+extern "C" int slab_rows(int format, int M, int nt) { return marlin_b200::tc_slab_rows(format, M, nt); }
 """
 
 
 @pytest.fixture(scope="module")
-def plan(tmp_path_factory):
+def shim(tmp_path_factory):
     d = tmp_path_factory.mktemp("plan")
     (d / "shim.cpp").write_text(SHIM)
     so = str(d / "shim.so")
     subprocess.run(["g++", "-O1", "-std=c++17", "-shared", "-fPIC", "-I", os.path.join(ROOT, "paper_2408_11743_b200", "csrc"),
                     str(d / "shim.cpp"), "-o", so], check=True)
-    L = ctypes.CDLL(so)
+    return ctypes.CDLL(so)
 
+
+@pytest.fixture(scope="module")
+def plan(shim):
     def ask(fmt, M, K, N, sms=148, most=160):
         out = (ctypes.c_longlong * 6)()
-        L.plan(fmt, M, K // 128, N, sms, most, out)
+        shim.plan(fmt, M, K // 128, N, sms, most, out)
         return dict(zip(("nt", "whole", "split", "cluster", "workers", "ncols"), out))
     return ask
 
@@ -94,3 +98,18 @@ def test_every_plan_can_run(plan, monkeypatch, fmt, env):
 def test_picks_among_the_fastest_of_the_timed_candidates(plan, fmt, M, K, N, good):
     p = plan(fmt, M, K, N)
     assert (p["nt"], p["split"] or ("whole" if p["whole"] else "even")) in good
+
+
+@pytest.mark.parametrize("fmt", [DENSE4, SPARSE4, DENSE8, DEFERRED4, ZERO4])
+def test_slabs_cover_every_batch(shim, fmt):
+    for M in list(range(1, 3000)) + [4095, 4096, 4097, 65535, 70000]:
+        mpad = 32 if M <= 32 else 64 if M <= 64 else 128
+        slabs = -(-M // mpad)
+        for nt in (1, 2):
+            rows = shim.slab_rows(fmt, M, nt)
+            assert rows % 16 == 0 and rows <= mpad  # the MMA's N; the instance's stages and accumulators
+            assert (slabs - 1) * rows < M <= slabs * rows  # all rows, no empty slab
+            # the heights that the issuers have loops for; the planner counts on one height for both tile widths where there are several slabs
+            assert rows in ({16, 32} if mpad == 32 else {64} if mpad == 64 else {80, 96, 112, 128})
+            assert rows == mpad or (fmt != DEFERRED4 and (mpad == 128 or (M <= 16 and nt == 2)))
+        assert slabs == 1 or shim.slab_rows(fmt, M, 1) == shim.slab_rows(fmt, M, 2)
