@@ -159,6 +159,13 @@ __device__ __forceinline__ void tc_ld_frag(uint32_t taddr, float* r) {
                : "r"(taddr)
                : "memory");
 }
+// the same, 8 columns: registers e
+__device__ __forceinline__ void tc_ld_frag8(uint32_t taddr, float* r) {
+  asm volatile("tcgen05.ld.sync.aligned.16x256b.x1.b32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3])
+               : "r"(taddr)
+               : "memory");
+}
 // 8 x 8 fragments of 16-bit values, transposed: lanes 8i .. 8i + 7 give the row addresses of matrix i
 __device__ __forceinline__ void stmatrix_x4_trans(uint32_t saddr, const uint32_t (&r)[4]) {
   asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(saddr), "r"(r[0]), "r"(r[1]),
@@ -486,20 +493,26 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
       sc[0] = s01.x; sc[1] = s01.y; sc[2] = s23.x; sc[3] = s23.y;
     }
   };
-  // 16 rows from row m on out of tensor memory, the halves of the k-blocks added, scaled: f[8b + 4h + e].  Every product and sum of the
-  // fix-up is rounded by itself (no fma): whether a CTA's part goes into the sum from registers or through a slot depends on who
-  // comes first and must not show.
-  auto load_rows = [&](int t, int m, const float (&sc)[4], float (&f)[16]) {
-    float a[2][8], a2[2][8];
+  // 8 NBK rows from row m on out of tensor memory, the halves of the k-blocks added, scaled: f[8b + 4h + e].  Every product and sum
+  // of the fix-up is rounded by itself (no fma): whether a CTA's part goes into the sum from registers or through a slot depends on
+  // who comes first and must not show.
+  auto load_rows = [&](auto nbk_c, int t, int m, const float (&sc)[4], float* f) {
+    constexpr int NBK = decltype(nbk_c)::value;
+    float a[2][4 * NBK], a2[2][4 * NBK];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const uint32_t at = tmem_base + ((quad * 32u + (uint32_t)(16 * h)) << 16) + (uint32_t)(t * KH * MPAD + m);
-      tc_ld_frag(at, a[h]);
-      if constexpr (KH == 2) tc_ld_frag(at + MPAD, a2[h]);
+      if constexpr (NBK == 2) {
+        tc_ld_frag(at, a[h]);
+        if constexpr (KH == 2) tc_ld_frag(at + MPAD, a2[h]);
+      } else {
+        tc_ld_frag8(at, a[h]);
+        if constexpr (KH == 2) tc_ld_frag8(at + MPAD, a2[h]);
+      }
     }
     tc_wait_ld();
 #pragma unroll
-    for (int x = 0; x < 16; ++x) {
+    for (int x = 0; x < 8 * NBK; ++x) {
       const int h = (x >> 2) & 1, i = 4 * (x >> 3) + (x & 3);
       f[x] = a[h][i];
       if constexpr (KH == 2) f[x] = __fadd_rn(f[x], a2[h][i]);
@@ -519,100 +532,112 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
     const int last_w = p.split ? (int)(vcol * p.split + p.split - 1) : (int)stripe_owner32((vcol + 1) * KB - 1, U, P);
     const bool shared_tile = !p.whole && last_w > first_w, clustered = p.cluster > 1;
     int* stripe_counter = &p.counters[(uint32_t)p.ncols <= P ? vcol : (uint32_t)first_w];
-    // what is in tensor memory of piece c
-    auto own_sums = [&](int c, float (&f)[16]) {
-      const int t = c % NT;
+    constexpr IntC<1> one{};
+    constexpr IntC<2> two{};
+    // NBK blocks of eight rows from block b on (of tile t) out of tensor memory
+    auto own_sums = [&](auto nbk_c, int t, int b, float* f) {
       float sc[4];
       column_scales(col, t, sc);
       mbar_wait(&dfull[t], phase, abort_flag, p.status);
       tc_fence_after_sync();
-      load_rows(t, c / NT * 16, sc, f);
+      load_rows(nbk_c, t, 8 * b, sc, f);
     };
-    // block y / 2 of the piece (rows), half y % 2 (channels), in a slot
-    auto piece_index = [&](int c, int y) { return frag_index((c % NT) * 4 + (int)quad, c / NT * 2 + (y >> 1), y & 1); };
-    auto in_rows = [&](int c, int y) { return c / NT * 16 + 8 * (y >> 1) < m_lim; };
-    auto to_slot = [&](int c, const float (&f)[16], float4* slot) {
+    // half y % 2 (channels) of block b + y / 2 in a slot
+    auto index_of = [&](int t, int b, int y) { return frag_index(t * 4 + (int)quad, b + (y >> 1), y & 1); };
+    auto has = [&](int b, int y) { return 8 * (b + (y >> 1)) < m_lim; };  // (its rows exist)
+    auto to_slot = [&](auto nbk_c, int t, int b, const float* f, float4* slot) {
 #pragma unroll
-      for (int y = 0; y < 4; ++y)
-        if (in_rows(c, y)) slot[piece_index(c, y)] = make_float4(f[4 * y], f[4 * y + 1], f[4 * y + 2], f[4 * y + 3]);
+      for (int y = 0; y < 2 * decltype(nbk_c)::value; ++y)
+        if (has(b, y)) slot[index_of(t, b, y)] = make_float4(f[4 * y], f[4 * y + 1], f[4 * y + 2], f[4 * y + 3]);
     };
-    auto to_c = [&](int c, const float (&f)[16]) {
-      const int c32 = (c % NT) * 4 + (int)quad;
+    auto to_c = [&](auto nbk_c, int t, int b, const float* f) {
+      const int c32 = t * 4 + (int)quad;
       if (col * G::TN + (uint32_t)c32 * 32 >= (uint32_t)p.N) return;
 #pragma unroll
-      for (int b = 0; b < 2; ++b) {
+      for (int i = 0; i < decltype(nbk_c)::value; ++i) {
         float fb[8];
 #pragma unroll
-        for (int x = 0; x < 8; ++x) fb[x] = f[8 * b + x];
-        store_block(c32, c / NT * 2 + b, fb, b, col, m_lim, row0);
+        for (int x = 0; x < 8; ++x) fb[x] = f[8 * i + x];
+        store_block(c32, b + i, fb, i, col, m_lim, row0);
       }
     };
-    // Piece c of n partial tiles in their order: tile `own` (n: none) from tensor memory, the others from their slots, three of them
-    // on their way at a time (a cluster of four: one latency of the L2), and cleared behind the read (a workspace comes back as it was given).
-    auto gather = [&](int c, int n, int own, auto slot, float (&sum)[16]) {
-      float f[16];
-      if (own < n) own_sums(c, f);
+    // Blocks of n partial tiles in their order: tile `own` (n: none) from tensor memory, the others from their slots, three of them
+    // on their way at a time (a cluster of four: one latency of the L2), and cleared behind the read (a workspace comes back as it was
+    // given; behind the stores of C, in a loop of its own, it takes 0.1 to 0.3 us longer).  The sums go to `to` or, without one, to C.
+    auto gather = [&](auto nbk_c, int t, int b, int n, int own, auto slot, float4* to) {
+      constexpr int NBK = decltype(nbk_c)::value;
+      float f[8 * NBK], sum[8 * NBK];
+      if (own < n) own_sums(nbk_c, t, b, f);
 #pragma unroll
-      for (int x = 0; x < 16; ++x) sum[x] = 0.f;
+      for (int x = 0; x < 8 * NBK; ++x) sum[x] = 0.f;
       const int others = own < n ? n - 1 : n;
       constexpr int UN = 3;
       for (int o = 0; o < others; o += UN) {
-        float4 v[UN][4];
+        float4 v[UN][2 * NBK];
         float4* from[UN];
 #pragma unroll
         for (int i = 0; i < UN; ++i)
           if (o + i < others) {
             from[i] = slot(o + i + (o + i >= own ? 1 : 0));
 #pragma unroll
-            for (int y = 0; y < 4; ++y)
-              if (in_rows(c, y)) v[i][y] = ld_cg_f4(from[i] + piece_index(c, y));
+            for (int y = 0; y < 2 * NBK; ++y)
+              if (has(b, y)) v[i][y] = ld_cg_f4(from[i] + index_of(t, b, y));
           }
 #pragma unroll
         for (int i = 0; i < UN; ++i)
           if (o + i < others) {
             if (o + i == own) {
 #pragma unroll
-              for (int x = 0; x < 16; ++x) sum[x] = __fadd_rn(sum[x], f[x]);
+              for (int x = 0; x < 8 * NBK; ++x) sum[x] = __fadd_rn(sum[x], f[x]);
             }
 #pragma unroll
-            for (int y = 0; y < 4; ++y)
-              if (in_rows(c, y)) {
+            for (int y = 0; y < 2 * NBK; ++y)
+              if (has(b, y)) {
                 sum[4 * y] = __fadd_rn(sum[4 * y], v[i][y].x); sum[4 * y + 1] = __fadd_rn(sum[4 * y + 1], v[i][y].y);
                 sum[4 * y + 2] = __fadd_rn(sum[4 * y + 2], v[i][y].z); sum[4 * y + 3] = __fadd_rn(sum[4 * y + 3], v[i][y].w);
-                from[i][piece_index(c, y)] = make_float4(0.f, 0.f, 0.f, 0.f);
+                from[i][index_of(t, b, y)] = make_float4(0.f, 0.f, 0.f, 0.f);
               }
           }
       }
       if (own == n - 1) {
 #pragma unroll
-        for (int x = 0; x < 16; ++x) sum[x] = __fadd_rn(sum[x], f[x]);
+        for (int x = 0; x < 8 * NBK; ++x) sum[x] = __fadd_rn(sum[x], f[x]);
       }
+      if (to)
+        to_slot(nbk_c, t, b, sum, to);
+      else
+        to_c(nbk_c, t, b, sum);
     };
     pdl_wait_prior_grids();
     float f[16];
     if (clustered) {
-      // CTAs of a split tile in clusters: the pieces are dealt out to them.  A CTA leaves those of the others in its slot and, behind the
-      // cluster barrier, adds the others' parts of its own pieces to what it has in tensor memory, in rank order.  (Through the L2 and not
+      // CTAs of a split tile in clusters: the tile is dealt out to them in units of 32 channels x 8 rows; unit c: tile c % NT, block
+      // c / NT, to rank c % cluster and warpgroup c / cluster % 4 of it.  A CTA leaves the units of the others in its slot and, behind the
+      // cluster barrier, adds the others' parts of its own units to what it has in tensor memory, in rank order.  (In whole pieces
+      // four CTAs with two tiles of 32 rows had four warps each at work, twice as long, and up to 16 rows two of them nothing to do:
+      // 8192 x 8192 at 24 / 32 / 64 rows 13.2 / 13.3 / 14.7 us so, 12.6 / 12.8 / 14.5 in units; 4096 x 4096 at 64 rows 8.7 / 7.9; 8-bit, four
+      // rows of 8192 x 8192 14.6 / 14.2; 2:4, 64 rows 11.9 / 11.7.  One body for all steps and partitions, its numbers in variables: half the
+      // code, and 1 to 10 % longer.  Through the L2 and not
       // through distributed shared memory: bulk copies from one shared memory into another, which exchange 32 KB among four CTAs in 2630
       // cycles instead of 4170, need a handshake before them and a barrier before a CTA may exit, and took 1 to 1.5 us longer in all.)
       const int cs = (int)p.cluster, C = (int)p.split / cs, r = (int)cluster_ctarank();
       float4* mine = slot_ptr(worker);
-      for (int c = g; c < pieces; c += 4)
-        if (c % cs != r) {
-          own_sums(c, f);
-          to_slot(c, f, mine);
-        }
-      cluster_sync_all();
-      const uint32_t first = worker - (uint32_t)r, shares = P + vcol * (uint32_t)C;
-      for (int c = r + cs * g; c < pieces; c += 4 * cs) {
-        gather(c, cs, r, [&](int q) { return slot_ptr(first + (uint32_t)q); }, f);
-        if (C == 1)
-          to_c(c, f);
-        else
-          to_slot(c, f, slot_ptr(shares + (worker / (uint32_t)cs) % (uint32_t)C));
+      for (int c = g; c < pieces; c += 4) {
+        const int t = c % NT, b = c / NT * 2;
+        const bool lo = (t + NT * b) % cs != r, hi = (t + NT * (b + 1)) % cs != r && has(b, 2);
+        if (!lo && !hi) continue;
+        own_sums(two, t, b, f);
+        if (lo) to_slot(one, t, b, f, mine);
+        if (hi) to_slot(one, t, b + 1, f + 8, mine);
       }
+      cluster_sync_all();
+      const int units = NT * ((m_lim + 7) >> 3);
+      const uint32_t first = worker - (uint32_t)r, shares = P + vcol * (uint32_t)C;
+      float4* share = C == 1 ? nullptr : slot_ptr(shares + (worker / (uint32_t)cs) % (uint32_t)C);
+      for (int c = r + cs * g; c < units; c += 4 * cs)
+        gather(one, c % NT, c / NT, cs, r, [&](int q) { return slot_ptr(first + (uint32_t)q); }, share);
       if (C == 1) return;
-      // the CTAs of rank r of the tile's clusters hold the same pieces: whoever of them comes last adds them up
+      // the CTAs of rank r of the tile's clusters hold the same units: whoever of them comes last adds them up
       named_bar_sync(1, kAuxWarp0 * 32);
       if (w16 == 0 && lane == 0) {
         int* counter = &p.counters[vcol * (uint32_t)cs + r];
@@ -622,10 +647,8 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
       }
       named_bar_sync(1, kAuxWarp0 * 32);
       if (*last_flag != 0)
-        for (int c = r + cs * g; c < pieces; c += 4 * cs) {
-          gather(c, C, C, [&](int q) { return slot_ptr(shares + (uint32_t)q); }, f);
-          to_c(c, f);
-        }
+        for (int c = r + cs * g; c < units; c += 4 * cs)
+          gather(one, c % NT, c / NT, C, C, [&](int q) { return slot_ptr(shares + (uint32_t)q); }, nullptr);
       return;
     }
     // Stripes.  Where the other CTAs of the tile have left their parts already (the usual case: it was their first tile), this one adds
@@ -634,14 +657,16 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
     named_bar_sync(1, kAuxWarp0 * 32);  // (also: the drain is done with the tile before, which went through all output buffers)
     const bool onto = *others_flag != 0;
     for (int c = g; c < pieces; c += 4) {
-      if (onto)
-        gather(c, last_w - first_w + 1, (int)worker - first_w, [&](int q) { return stripe_slot(first_w + q, vcol); }, f);
-      else
-        own_sums(c, f);
-      if (shared_tile && !onto)
-        to_slot(c, f, stripe_slot((int)worker, vcol));
-      else
-        to_c(c, f);
+      const int t = c % NT, b = c / NT * 2;
+      if (onto) {
+        gather(two, t, b, last_w - first_w + 1, (int)worker - first_w, [&](int q) { return stripe_slot(first_w + q, vcol); }, nullptr);
+      } else {
+        own_sums(two, t, b, f);
+        if (shared_tile)
+          to_slot(two, t, b, f, stripe_slot((int)worker, vcol));
+        else
+          to_c(two, t, b, f);
+      }
     }
     if (onto) {
       if (w16 == 0 && lane == 0) *stripe_counter = 0;
@@ -1220,10 +1245,10 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
           mbar_wait(&dfull[t], seg & 1u, abort_flag, p.status);
           tc_fence_after_sync();
           if (part) {
-#pragma unroll 2
+#pragma unroll 1  // (by two: 184 bytes of spills in the instance of 64 rows with one scale per column)
             for (int m = 0; m < MPAD; m += 16) {
               float f[16];
-              load_rows(t, m, sc, f);
+              load_rows(IntC<2>{}, t, m, sc, f);
               if (m + 16 == MPAD) release(t);
 #pragma unroll
               for (int b = 0; b < 2; ++b)
@@ -1241,7 +1266,7 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
 #pragma unroll
             for (int m = 0; m < MPAD; m += 16) {
               float f[16];
-              load_rows(t, m, sc, f);
+              load_rows(IntC<2>{}, t, m, sc, f);
 #pragma unroll
               for (int b = 0; b < 2; ++b) {
                 const int x = m / 8 + b;

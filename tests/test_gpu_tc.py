@@ -183,3 +183,56 @@ def test_scaled_parts_are_rounded_and_added_in_worker_order(marlin, monkeypatch,
         torch.cuda.synchronize()
         assert marlin.read_status(layer.ws) == 0
         assert torch.equal(C, want), int((C != want).sum())
+
+
+# Every format at the edges of slabs, units of eight rows and instances, in clusters of every size, stripes and k-ranges without
+# clusters.  Small integers times powers of two: every partial sum is exact, in any order.
+@pytest.mark.parametrize("tile", ["128", "256"])
+@pytest.mark.parametrize("fmt", ["column", "group", "zp", "sub", "w8", "w8-column", "sparse24", "sparse24-sub", "swiglu"])
+def test_every_format_at_every_height_and_cluster_size(marlin, monkeypatch, fmt, tile):
+    import torch
+    monkeypatch.setenv("MARLIN_B200_TC_TILE", tile)
+    K, N = 1024, 512
+    G = K if "column" in fmt else 64 if "sub" in fmt else 128
+    rng = np.random.default_rng(len(fmt))
+    s = np.ldexp(1.0, rng.integers(-6, -2, size=(K // G, N))).astype(np.float16)
+    S = np.repeat(s.astype(np.float64), G, axis=0)
+    ws = marlin.new_workspace(400, K, N)
+    if "w8" in fmt:
+        Q = rng.integers(0, 256, size=(K, N), dtype=np.uint8)
+        W = (Q - 128.0) * S
+        layer = marlin.Layer(*marlin.pack_w8(to_dev(Q), to_dev(s), G), K, N, G, ws, w8=True)
+    elif "sparse24" in fmt:
+        case = inputs.make_sparse24(1, K, N, G, seed=3)
+        codes = np.stack([(case.qc_kpacked >> np.uint32(4 * j)) & 15 for j in range(8)], axis=1).reshape(K // 2, N)
+        W = np.zeros((K, N))
+        np.put_along_axis(W.reshape(K // 4, 4, N), case.idx.reshape(K // 4, 2, N).astype(np.int64), codes.reshape(K // 4, 2, N) - 8.0, axis=1)
+        W *= S
+        w, meta, sp = marlin.pack_sparse24(to_dev(case.qc_kpacked), to_dev(case.idx), to_dev(s), G)
+        layer = marlin.Layer(w, sp, K, N, G, ws, meta_packed=meta)
+    else:
+        Q = rng.integers(0, 16, size=(K, N), dtype=np.uint8)
+        Z = rng.integers(0, 16, size=(K // G, N), dtype=np.uint8) if fmt == "zp" else np.full((K // G, N), 8, np.uint8)
+        W = (Q - np.repeat(Z.astype(np.float64), G, axis=0)) * S
+        packed = marlin.pack(to_dev(inputs.kpack(Q)), to_dev(s), G)
+        z = {"z_packed": marlin.pack_zeros(to_dev(Z), K, N, G)} if fmt == "zp" else {}
+        layer = marlin.Layer(*packed, K, N, G, ws, **z)
+    W = torch.from_numpy(W).cuda()
+    first = 17 if fmt in ("column", "group", "zp", "swiglu") else 1  # (below that the warp-level kernel)
+    for M in [m for m in (1, 8, 9, 15, 16, 17, 24, 25, 32, 33, 40, 48, 49, 64, 65, 72, 80, 81, 97, 112, 113, 128, 130, 161, 225, 300) if m >= first]:
+        A = to_dev(rng.integers(-2, 3, size=(M, K)).astype(np.float16))
+        want = (A.double() @ W).half()
+        for split, cluster in [(2, 8), (3, 8), (4, 8), (5, 8), (6, 8), (7, 8), (8, 8), (4, 2), (6, 3), (6, 2), (8, 4), (3, 0), (0, 0), (1, 8)]:
+            monkeypatch.setenv("MARLIN_B200_TC_SPLIT", str(split))
+            monkeypatch.setenv("MARLIN_B200_TC_CLUSTER", str(cluster))
+            if fmt == "swiglu":
+                H = marlin.gemm_swiglu(A, *packed, K, N, G, ws)
+                c = want.double().view(M, N // 16, 2, 8)
+                g, u = c[:, :, 0].reshape(M, N // 2), c[:, :, 1].reshape(M, N // 2)
+                h = g / (1 + torch.exp(-g)) * u  # the bound of test_fused_activation_on_the_way_out
+                assert bool(((H.double() - h).abs() <= 2.0 ** -10.9 * h.abs() + 2.0 ** -25 + 1e-9).all()), (M, split, cluster)
+            else:
+                assert torch.equal(layer(A), want), (M, split, cluster)
+    torch.cuda.synchronize()
+    assert marlin.read_status(ws) == 0
+    assert bool((ws[256:] == 0).all())
