@@ -16,7 +16,7 @@
 // what runs in parallel.
 //   - Groups of 32, 64 or 128 rows: one thread owns one (group, column) and holds its rows in registers, one read of W.
 //   - Longer groups (up to one scale per column): three launches.  Column maxima in parts of 128 rows; then the search
-//     with one thread per (column, candidate), so that the serial sum over the rows runs for all candidates at
+//     with one thread per column and one or two candidates, so that the serial sum over the rows runs for all candidates at
 //     once; then the codes, parallel over the rows.  (One thread per column, which re-read the group once per candidate,
 //     left the chip idle on such layers: 4096 x 4096 with one scale per column took 7.96 ms.)
 // Only |w_i - (q_i - 8) s_t| enters e_t, and that leaves the search a freedom: where w_i / s_t lies half way between two codes both
@@ -26,7 +26,7 @@
 //   u = sat(w / (15 s) + 8 / 15),   q = round(15 u)        (error below 2^-18 codes)
 // the saturation of the first fma to [0, 1] is the clamp to [0, 15].  The codes themselves are made as written above.
 // Bound: the fp32 pipe, five operations per weight and candidate (u, two for the rounding, two for the error), most of them issued in
-// pairs (fma.rn.f32x2 and the like: the same IEEE operations, half the instructions); no conversions, no comparisons.
+// pairs (fma.rn.f32x2 and the like: the same IEEE operations, half the instructions); no conversions to integers, no comparisons.
 // Measured with ten candidates, before (clamp by two comparisons) and now: 4096 x 11008, groups of 128: 114 / 99 us; one scale per column,
 // 4096 x 4096: 99 / 85, 8192 x 1024: 163 / 134.
 #include "device_utils.cuh"
@@ -167,14 +167,104 @@ quantize_max_kernel(const uint16_t* __restrict__ W, uint32_t* __restrict__ q_kpa
   reinterpret_cast<uint2*>(q_kpacked + (size_t)part * (kPartRows / 8) * N)[n2] = make_uint2(m & 0xffffu, m >> 16);
 }
 
-// The search: lane = column, warp = one candidate, rows in order.  The rows come through a ring of shared-memory tiles (64 rows x 32
-// columns, three tiles ahead): with few warps per scheduler nothing else hides the latency of the L2.  A tile is turned into
-// fp32 pairs of rows once for all candidates, one tile ahead of the sums.
+// The search: lane = column, rows in order, a warp one candidate or a pair of them.  The rows come through a ring of shared-memory tiles
+// (64 rows x 32 columns, three tiles ahead): with few warps per scheduler nothing else hides the latency of the L2.
 constexpr int kSearchCols = 32, kSearchMinWarps = 8, kSearchMaxWarps = 16, kSearchRows = 64, kSearchTiles = 4;
+typedef uint16_t SearchRing[kSearchTiles][kSearchRows][kSearchCols];
+// asks for tile `tile` of the columns from w on, if it is one; one group of copies per call, empty ones too
+__device__ __forceinline__ void fetch_tile(SearchRing& ring, const uint16_t* w, int N, int tile, int tiles) {
+  if (tile < tiles) {
+    for (int v = threadIdx.x; v < kSearchRows * 4; v += blockDim.x) {
+      const int row = v >> 2, part = v & 3;
+      const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&ring[tile % kSearchTiles][row][8 * part]);
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(w + ((size_t)tile * kSearchRows + row) * N + 8 * part)
+                   : "memory");
+    }
+  }
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+// the largest weight of a group, from the maxima of its parts
+__device__ __forceinline__ float group_max(const uint32_t* q_kpacked, int N, int G, int g, int n) {
+  uint32_t amax = 0;
+  for (int part = 0; part < G / kPartRows; ++part)
+    amax = max(amax, __ldg(q_kpacked + ((size_t)g * (G / kPartRows) + part) * (kPartRows / 8) * N + n));
+  return __half2float(__ushort_as_half((uint16_t)amax));
+}
+
+// Warp = PER candidates (in the halves of a register pair), rows straight out of the ring.
+template <int PER>
+__global__ void __launch_bounds__(kSearchCols * kSearchMaxWarps)
+quantize_search_direct_kernel(const uint16_t* __restrict__ W, const uint32_t* __restrict__ q_kpacked, uint16_t* __restrict__ scales,
+                              int N, int G, int n_grid, int n_candidates) {
+  __shared__ __align__(16) SearchRing ring;
+  __shared__ float errs[PER * kSearchMaxWarps][kSearchCols];
+  __shared__ uint16_t cands[PER * kSearchMaxWarps][kSearchCols];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  const int n = blockIdx.x * kSearchCols + lane;
+  const int g = blockIdx.y;
+  const uint16_t* w = W + (size_t)g * G * N + blockIdx.x * kSearchCols;
+  const int tiles = G / kSearchRows;  // G is a multiple of 128
+  const float a = group_max(q_kpacked, N, G, g, n);
+  const f32x2 magic = pack2(kRoundMagic, kRoundMagic), minus_magic8 = pack2(-kRoundMagic - 8.f, -kRoundMagic - 8.f);
+  const f32x2 fifteen = pack2(15.f, 15.f);
+  float best_err = __int_as_float(0x7f800000);
+  uint16_t best_s = 1;
+  for (int t0 = 0; t0 < n_candidates; t0 += PER * warps) {
+    // (slots past the last candidate repeat it)
+    float s[PER], inv15[PER], err[PER];
+#pragma unroll
+    for (int c = 0; c < PER; ++c) {
+      cands[PER * warp + c][lane] = candidate_scale(a, min(t0 + PER * warp + c, n_candidates - 1), n_grid, s[c], inv15[c]);
+      err[c] = 0.f;
+    }
+    f32x2 err2 = pack2(0.f, 0.f);
+    for (int i = 0; i < kSearchTiles - 1; ++i) fetch_tile(ring, w, N, i, tiles);
+    for (int tile = 0; tile < tiles; ++tile) {
+      asm volatile("cp.async.wait_group %0;" ::"n"(kSearchTiles - 2) : "memory");
+      __syncthreads();  // this tile has landed for everybody, and everybody has left the one before it
+      fetch_tile(ring, w, N, tile + kSearchTiles - 1, tiles);
+      const uint16_t* rows = &ring[tile % kSearchTiles][0][lane];
+#pragma unroll 16
+      for (int i = 0; i < kSearchRows; ++i) {
+        const float x = __half2float(__ushort_as_half(rows[i * kSearchCols]));
+        if constexpr (PER == 2) {
+          float q[2];
+          const f32x2 y = fma2(pack2(unit_of(x, inv15[0]), unit_of(x, inv15[1])), fifteen, magic);  // magic + q + 8
+          unpack2(add2(y, minus_magic8), q[0], q[1]);
+          const f32x2 d = pack2(__fmaf_rn(-q[0], s[0], x), __fmaf_rn(-q[1], s[1], x));
+          err2 = fma2(d, d, err2);
+        } else {
+          const float q = __fsub_rn(__fmaf_rn(unit_of(x, inv15[0]), 15.f, kRoundMagic), kRoundMagic + 8.f);
+          const float d = __fmaf_rn(-q, s[0], x);
+          err[0] = __fmaf_rn(d, d, err[0]);
+        }
+      }
+    }
+    if constexpr (PER == 2) unpack2(err2, err[0], err[1]);
+#pragma unroll
+    for (int c = 0; c < PER; ++c) errs[PER * warp + c][lane] = err[c];
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    if (warp == 0) {
+      // in candidate order, the first one on ties
+      for (int c = 0; c < PER * warps && t0 + c < n_candidates; ++c)
+        if (errs[c][lane] < best_err) {
+          best_err = errs[c][lane];
+          best_s = cands[c][lane];
+        }
+    }
+    __syncthreads();
+  }
+  if (warp == 0) scales[(size_t)g * N + n] = best_s;
+}
+
+// Warp = one candidate; a tile is turned into fp32 pairs of rows once for all candidates, one tile ahead of the sums.  IDLE: warps without
+// a candidate fetch and widen only (else they repeat the last one: a branch around the sums takes 6 % longer).
+template <bool IDLE>
 __global__ void __launch_bounds__(kSearchCols * kSearchMaxWarps)
 quantize_search_kernel(const uint16_t* __restrict__ W, const uint32_t* __restrict__ q_kpacked, uint16_t* __restrict__ scales,
                        int N, int G, int n_grid, int n_candidates) {
-  __shared__ __align__(16) uint16_t ring[kSearchTiles][kSearchRows][kSearchCols];
+  __shared__ __align__(16) SearchRing ring;
   __shared__ f32x2 pairs[2][kSearchRows / 2][kSearchCols];
   __shared__ float errs[kSearchMaxWarps][kSearchCols];
   __shared__ uint16_t cands[kSearchMaxWarps][kSearchCols];
@@ -183,18 +273,7 @@ quantize_search_kernel(const uint16_t* __restrict__ W, const uint32_t* __restric
   const int g = blockIdx.y;
   const uint16_t* w = W + (size_t)g * G * N + blockIdx.x * kSearchCols;
   const int tiles = G / kSearchRows;  // G is a multiple of 128
-  auto fetch = [&](int tile) {
-    if (tile < tiles) {
-      for (int v = threadIdx.x; v < kSearchRows * 4; v += blockDim.x) {
-        const int row = v >> 2, part = v & 3;
-        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&ring[tile % kSearchTiles][row][8 * part]);
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst),
-                     "l"(w + ((size_t)tile * kSearchRows + row) * N + 8 * part)
-                     : "memory");
-      }
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");  // one group per call, empty ones too
-  };
+  auto fetch = [&](int tile) { fetch_tile(ring, w, N, tile, tiles); };
   // rows of a tile from 16 to 32 bits, in two steps: loads into registers, and later their way into `pairs`
   constexpr int kWiden = kSearchRows / 2 / kSearchMinWarps;
   uint16_t wide[kWiden][2];
@@ -216,16 +295,13 @@ quantize_search_kernel(const uint16_t* __restrict__ W, const uint32_t* __restric
         pairs[tile & 1][r2][lane] = pack2(__half2float(__ushort_as_half(wide[i][0])), __half2float(__ushort_as_half(wide[i][1])));
     }
   };
-  uint32_t amax = 0;
-  for (int part = 0; part < G / kPartRows; ++part)
-    amax = max(amax, __ldg(q_kpacked + ((size_t)g * (G / kPartRows) + part) * (kPartRows / 8) * N + n));
-  const float a = __half2float(__ushort_as_half((uint16_t)amax));
+  const float a = group_max(q_kpacked, N, G, g, n);
   const f32x2 magic = pack2(kRoundMagic, kRoundMagic), magic8 = pack2(kRoundMagic + 8.f, kRoundMagic + 8.f);
   const f32x2 minus1 = pack2(-1.f, -1.f), fifteen = pack2(15.f, 15.f);
   float best_err = __int_as_float(0x7f800000);
   uint16_t best_s = 1;
   for (int t0 = 0; t0 < n_candidates; t0 += warps) {
-    // (warps past the last candidate repeat it)
+    const bool mine = !IDLE || t0 + warp < n_candidates;
     constexpr int B = 4;
     float s, inv15, err = 0.f, d[2 * B];
 #pragma unroll
@@ -247,35 +323,37 @@ quantize_search_kernel(const uint16_t* __restrict__ W, const uint32_t* __restric
       // Four pairs at a time, each operation for all of them, the next four already on their way and the squares of the four
       // before (a chain, in row order) in between: with two or three warps per scheduler one after the other would wait for itself
       // (two, four, eight at a time: 91, 85, 85 us for 4096 x 4096 with one scale per column; 167, 157, 169 for 4096 x 11008 in groups of 256).
-      f32x2 next[B];
+      if (mine) {
+        f32x2 next[B];
 #pragma unroll
-      for (int i = 0; i < B; ++i) next[i] = rows[i * kSearchCols];
+        for (int i = 0; i < B; ++i) next[i] = rows[i * kSearchCols];
 #pragma unroll
-      for (int i0 = 0; i0 < kSearchRows / 2; i0 += B) {
-        f32x2 ww[B], y[B];
-        float u[2 * B];
+        for (int i0 = 0; i0 < kSearchRows / 2; i0 += B) {
+          f32x2 ww[B], y[B];
+          float u[2 * B];
 #pragma unroll
-        for (int i = 0; i < B; ++i) {
-          ww[i] = next[i];
-          if (i0 + B < kSearchRows / 2) next[i] = rows[(i0 + B + i) * kSearchCols];
+          for (int i = 0; i < B; ++i) {
+            ww[i] = next[i];
+            if (i0 + B < kSearchRows / 2) next[i] = rows[(i0 + B + i) * kSearchCols];
+          }
+#pragma unroll
+          for (int i = 0; i < B; ++i) {
+            float lo, hi;
+            unpack2(ww[i], lo, hi);
+            u[2 * i] = unit_of(lo, inv15);
+            u[2 * i + 1] = unit_of(hi, inv15);
+            err = __fmaf_rn(d[i], d[i], err);
+          }
+#pragma unroll
+          for (int i = 0; i < B; ++i) {
+            y[i] = fma2(pack2(u[2 * i], u[2 * i + 1]), fifteen, magic);  // magic + q + 8
+            err = __fmaf_rn(d[B + i], d[B + i], err);
+          }
+#pragma unroll
+          for (int i = 0; i < B; ++i) y[i] = fma2(y[i], minus1, magic8);  // -q, exactly
+#pragma unroll
+          for (int i = 0; i < B; ++i) unpack2(fma2(y[i], s2, ww[i]), d[2 * i], d[2 * i + 1]);
         }
-#pragma unroll
-        for (int i = 0; i < B; ++i) {
-          float lo, hi;
-          unpack2(ww[i], lo, hi);
-          u[2 * i] = unit_of(lo, inv15);
-          u[2 * i + 1] = unit_of(hi, inv15);
-          err = __fmaf_rn(d[i], d[i], err);
-        }
-#pragma unroll
-        for (int i = 0; i < B; ++i) {
-          y[i] = fma2(pack2(u[2 * i], u[2 * i + 1]), fifteen, magic);  // magic + q + 8
-          err = __fmaf_rn(d[B + i], d[B + i], err);
-        }
-#pragma unroll
-        for (int i = 0; i < B; ++i) y[i] = fma2(y[i], minus1, magic8);  // -q, exactly
-#pragma unroll
-        for (int i = 0; i < B; ++i) unpack2(fma2(y[i], s2, ww[i]), d[2 * i], d[2 * i + 1]);
       }
       if (tile + 1 < tiles) widen_store(tile + 1);
     }
@@ -338,9 +416,28 @@ cudaError_t launch_quantize_rtn(const uint16_t* W, uint32_t* q_kpacked, uint16_t
     const unsigned pairs = (unsigned)((N / 2 + 127) / 128);
     quantize_max_kernel<<<dim3(pairs, (unsigned)(K / kPartRows)), 128, 0, stream>>>(W, q_kpacked, N);
     const dim3 blocks((unsigned)(N / kSearchCols), (unsigned)(K / G));
-    // (warps without a candidate of their own fetch and widen all the same)
-    const int warps = n_candidates < kSearchMinWarps ? kSearchMinWarps : n_candidates < kSearchMaxWarps ? n_candidates : kSearchMaxWarps;
-    quantize_search_kernel<<<blocks, kSearchCols * warps, 0, stream>>>(W, q_kpacked, scales, N, G, n_grid, n_candidates);
+    // Pairs of candidates straight out of the ring take fewer instructions; single ones on widened rows spread over more warps and
+    // shorten the chains, as long as one round of warps takes them and few blocks share an SM.  Of 9 to 12 candidates the fullest of the
+    // four schedulers has four in pairs and three of single ones, of 13 to 16 four either way.  Measured, pairs / single, us: 4096 x 4096 with
+    // one scale per column (128 blocks) 8, 10, 16, 17 candidates 88.6 / 70.2, 102.9 / 84.5, 102.9 / 100.9, 127 / 141; 8192 x 1024 in groups of 1024
+    // (256) 50.3 / 45.5, 53.8 / 55.8 (10, 16); 4096 x 2048 in groups of 256 (1024) 35.3 / 35.3, 41.3 / 39.4, 49.6 / 51.7 (8, 10, 16); 4096 x 4096
+    // in groups of 256 (2048) 64.0 / 66.0 (10); 4096 x 11008 (5504) 80.6 / 134, 92.9 / 134, 150 / 156, 246 / 263 (1, 4, 10, 20).
+    const long long all = (long long)blocks.x * blocks.y;
+    const bool single = n_candidates <= kSearchMaxWarps && (all < 2 * 148 || (all < 2048 && n_candidates > 8 && n_candidates <= 12));
+    if (single && n_candidates > 4) {
+      const int warps = n_candidates < kSearchMinWarps ? kSearchMinWarps : n_candidates;
+      quantize_search_kernel<false><<<blocks, kSearchCols * warps, 0, stream>>>(W, q_kpacked, scales, N, G, n_grid, n_candidates);
+    } else if (single) {
+      // (up to four candidates: eight warps of which some have none, 64 us on 128 blocks and 30 to 33 on 256; all eight adding 70 and 39)
+      quantize_search_kernel<true><<<blocks, kSearchCols * kSearchMinWarps, 0, stream>>>(W, q_kpacked, scales, N, G, n_grid, n_candidates);
+    } else if (n_candidates == 1) {
+      quantize_search_direct_kernel<1><<<blocks, kSearchCols, 0, stream>>>(W, q_kpacked, scales, N, G, n_grid, n_candidates);
+    } else {
+      // rounds of equal size
+      const int pairs_all = (n_candidates + 1) / 2, rounds = (pairs_all + kSearchMaxWarps - 1) / kSearchMaxWarps;
+      quantize_search_direct_kernel<2><<<blocks, kSearchCols * ((pairs_all + rounds - 1) / rounds), 0, stream>>>(W, q_kpacked, scales, N, G,
+                                                                                                               n_grid, n_candidates);
+    }
     // one grid row per eight rows of W: up to 2^20 / 8, above the limit of grid.y, so the rows go on in slices of it
     constexpr int kSlice = 32768;
     for (int r0 = 0; r0 < K / 8; r0 += kSlice) {

@@ -52,6 +52,16 @@ def test_long_groups_match_the_oracle_bit_for_bit(marlin, K, N, G, n_grid, n_can
     test_codes_and_scales_match_the_oracle_bit_for_bit(marlin, K, N, G, n_grid, n_cand)
 
 
+# the forms of the search, by blocks (few, some, many) and candidates: none and some warps without a candidate, pairs with a last one
+# alone, rounds of equal and unequal size
+@pytest.mark.parametrize("K,N,G", [(1024, 64, 256), (1024, 128, -1), (2048, 1280, 256), (4096, 4096, 256)])
+@pytest.mark.parametrize("n_cand", [1, 2, 3, 4, 5, 7, 8, 9, 12, 13, 16, 17, 20, 32, 33, 50])
+def test_every_form_of_the_search_matches_the_oracle_bit_for_bit(marlin, K, N, G, n_cand):
+    if K * N > 1 << 22 and n_cand not in (1, 2, 9, 16, 33):
+        return
+    test_codes_and_scales_match_the_oracle_bit_for_bit(marlin, K, N, G, max(20, n_cand), n_cand)
+
+
 # weights half way between two codes, subnormals and the largest values: the search may take either code of a tie, the codes may not
 @pytest.mark.parametrize("G", [32, 64, 128, 256])
 @pytest.mark.parametrize("kind", ["halves", "subnormal", "largest", "wide"])
