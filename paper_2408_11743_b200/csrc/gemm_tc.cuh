@@ -1246,10 +1246,10 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
           tc_fence_after_sync();
           if (part) {
 #pragma unroll 1  // (by two: 184 bytes of spills in the instance of 64 rows with one scale per column)
-            for (int m = 0; m < MPAD; m += 16) {
+            for (int m = 0; m < (int)slab_rows; m += 16) {
               float f[16];
               load_rows(IntC<2>{}, t, m, sc, f);
-              if (m + 16 == MPAD) release(t);
+              if (m + 16 >= (int)slab_rows) release(t);
 #pragma unroll
               for (int b = 0; b < 2; ++b)
                 if (m + 8 * b < m_lim)
@@ -1265,6 +1265,7 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
             uint32_t rest[REST > 0 ? REST : 1][4];
 #pragma unroll
             for (int m = 0; m < MPAD; m += 16) {
+              if (MPAD == 128 && m >= (int)slab_rows) break;  // (what no MMA has written; what is put away of it is not stored)
               float f[16];
               load_rows(IntC<2>{}, t, m, sc, f);
 #pragma unroll

@@ -11,7 +11,7 @@ enum TcFormat { kTcDense4 = 0, kTcSparse4 = 1, kTcDense8 = 2, kTcDeferred4 = 3, 
 // the kernel's instance: the most rows that a slab of it has
 inline int tc_mpad(int m) { return m <= 32 ? 32 : (m <= 64 ? 64 : 128); }
 
-// Rows of a slab, the MMA's N.  From 65 rows on a batch is cut into equal slabs, in units of 16 rows: what MMAs and copies cost goes with the
+// Rows of a slab, the MMA's N.  From 65 rows on a batch is cut into equal slabs, in units of 16 rows: what MMAs, copies and read-out cost goes with the
 // rows of a slab, so 130 rows are two slabs of 80, not of 128 (8192 x 8192 at 130 rows 25.1 us so, 24.1 now; 4096 x 22016 at 100 rows
 // 25.6 / 24.6; 2:4, 4096 x 4096 at 300 rows 12.6 / 12.2).  Up to 16 rows on tiles of 256 columns a slab has 16 (28672 x 8192 with one scale per
 // column 25.6 us with 32, 25.3 so; 2:4, 8192 x 8192 at four rows 10.3 / 9.7).  The others are as high as the instance: rows that the issuer has
