@@ -409,7 +409,7 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
     return slot_ptr((uint32_t)(2 * w + ((!p.split && vcol != stripe_begin32((uint32_t)w, U, P) / KB) ? 1 : 0)));
   };
 
-  // Split tile, CTAs in clusters: every CTA has left its partial tile in its slot.  Behind the cluster barrier a CTA adds up
+  // Split tile, CTAs in clusters (deferred scales; the others: drain_last): every CTA has left its partial tile in its slot.  Behind the cluster barrier a CTA adds up
   // its share of the (32 channels, eight rows) blocks over the cluster, in rank order, and stores that part of C; where a
   // tile has several clusters the share goes to the cluster's slot and the last of them adds the shares in order.
   // (Through the L2 and not through distributed shared memory, which moves about 12 bytes per clock and SM here against
@@ -449,7 +449,7 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
       sum_blocks(x0, step, items, nb, col, C, [&](int q) { return slot_ptr(shares + (uint32_t)q); }, to_c);
   };
 
-  // Stripes, the last segment of a CTA: its partial tile is in its slot; the last arriver at the tile adds all of them up, all
+  // Stripes, the last segment of a CTA (deferred scales, likewise): its partial tile is in its slot; the last arriver at the tile adds all of them up, all
   // converting and draining warps together (they are done, and nothing else is left to hide the loads behind).
   // One counter per virtual column tile; where there are more of those than workers, per tile that can be shared, numbered by
   // the first worker on it (at most one tile runs over the end of a worker's stripe).
@@ -527,7 +527,7 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
     const uint32_t phase = (vcol - u0 / KB) & 1u;
     const size_t row0 = (size_t)slab * slab_rows;
     const int m_lim = min(p.M - (int)row0, (int)slab_rows);
-    const int pieces = NT * ((m_lim + 15) >> 4), g = w16 >> 2;
+    const int pieces = NT * ((m_lim + 15) >> 4), units = NT * ((m_lim + 7) >> 3), g = w16 >> 2;
     const int first_w = p.split ? (int)(vcol * p.split) : (int)stripe_owner32(vcol * KB, U, P);
     const int last_w = p.split ? (int)(vcol * p.split + p.split - 1) : (int)stripe_owner32((vcol + 1) * KB - 1, U, P);
     const bool shared_tile = !p.whole && last_w > first_w, clustered = p.cluster > 1;
@@ -561,26 +561,25 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
         store_block(c32, b + i, fb, i, col, m_lim, row0);
       }
     };
-    // Blocks of n partial tiles in their order: tile `own` (n: none) from tensor memory, the others from their slots, three of them
+    // Block b of n partial tiles in their order: tile `own` (n: none) from tensor memory, the others from their slots, three of them
     // on their way at a time (a cluster of four: one latency of the L2), and cleared behind the read (a workspace comes back as it was
     // given; behind the stores of C, in a loop of its own, it takes 0.1 to 0.3 us longer).  The sums go to `to` or, without one, to C.
-    auto gather = [&](auto nbk_c, int t, int b, int n, int own, auto slot, float4* to) {
-      constexpr int NBK = decltype(nbk_c)::value;
-      float f[8 * NBK], sum[8 * NBK];
-      if (own < n) own_sums(nbk_c, t, b, f);
+    auto gather = [&](int t, int b, int n, int own, auto slot, float4* to) {
+      float f[8], sum[8];
+      if (own < n) own_sums(one, t, b, f);
 #pragma unroll
-      for (int x = 0; x < 8 * NBK; ++x) sum[x] = 0.f;
+      for (int x = 0; x < 8; ++x) sum[x] = 0.f;
       const int others = own < n ? n - 1 : n;
       constexpr int UN = 3;
       for (int o = 0; o < others; o += UN) {
-        float4 v[UN][2 * NBK];
+        float4 v[UN][2];
         float4* from[UN];
 #pragma unroll
         for (int i = 0; i < UN; ++i)
           if (o + i < others) {
             from[i] = slot(o + i + (o + i >= own ? 1 : 0));
 #pragma unroll
-            for (int y = 0; y < 2 * NBK; ++y)
+            for (int y = 0; y < 2; ++y)
               if (has(b, y)) v[i][y] = ld_cg_f4(from[i] + index_of(t, b, y));
           }
 #pragma unroll
@@ -588,11 +587,11 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
           if (o + i < others) {
             if (o + i == own) {
 #pragma unroll
-              for (int x = 0; x < 8 * NBK; ++x) sum[x] = __fadd_rn(sum[x], f[x]);
+              for (int x = 0; x < 8; ++x) sum[x] = __fadd_rn(sum[x], f[x]);
             }
 #pragma unroll
-            for (int y = 0; y < 2 * NBK; ++y)
-              if (has(b, y)) {
+            for (int y = 0; y < 2; ++y)
+              if (has(b, y)) {  // (always so here; without the condition the loop is compiled to 1 to 4 % longer launches)
                 sum[4 * y] = __fadd_rn(sum[4 * y], v[i][y].x); sum[4 * y + 1] = __fadd_rn(sum[4 * y + 1], v[i][y].y);
                 sum[4 * y + 2] = __fadd_rn(sum[4 * y + 2], v[i][y].z); sum[4 * y + 3] = __fadd_rn(sum[4 * y + 3], v[i][y].w);
                 from[i][index_of(t, b, y)] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -601,12 +600,12 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
       }
       if (own == n - 1) {
 #pragma unroll
-        for (int x = 0; x < 8 * NBK; ++x) sum[x] = __fadd_rn(sum[x], f[x]);
+        for (int x = 0; x < 8; ++x) sum[x] = __fadd_rn(sum[x], f[x]);
       }
       if (to)
-        to_slot(nbk_c, t, b, sum, to);
+        to_slot(one, t, b, sum, to);
       else
-        to_c(nbk_c, t, b, sum);
+        to_c(one, t, b, sum);
     };
     pdl_wait_prior_grids();
     float f[16];
@@ -631,11 +630,10 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
         if (hi) to_slot(one, t, b + 1, f + 8, mine);
       }
       cluster_sync_all();
-      const int units = NT * ((m_lim + 7) >> 3);
       const uint32_t first = worker - (uint32_t)r, shares = P + vcol * (uint32_t)C;
       float4* share = C == 1 ? nullptr : slot_ptr(shares + (worker / (uint32_t)cs) % (uint32_t)C);
       for (int c = r + cs * g; c < units; c += 4 * cs)
-        gather(one, c % NT, c / NT, cs, r, [&](int q) { return slot_ptr(first + (uint32_t)q); }, share);
+        gather(c % NT, c / NT, cs, r, [&](int q) { return slot_ptr(first + (uint32_t)q); }, share);
       if (C == 1) return;
       // the CTAs of rank r of the tile's clusters hold the same units: whoever of them comes last adds them up
       named_bar_sync(1, kAuxWarp0 * 32);
@@ -648,30 +646,38 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
       named_bar_sync(1, kAuxWarp0 * 32);
       if (*last_flag != 0)
         for (int c = r + cs * g; c < units; c += 4 * cs)
-          gather(one, c % NT, c / NT, C, C, [&](int q) { return slot_ptr(shares + (uint32_t)q); }, nullptr);
+          gather(c % NT, c / NT, C, C, [&](int q) { return slot_ptr(shares + (uint32_t)q); }, nullptr);
       return;
     }
-    // Stripes.  Where the other CTAs of the tile have left their parts already (the usual case: it was their first tile), this one adds
-    // them to what it has and writes C; otherwise it leaves its own, and the last arriver adds up all of them.
+    // Stripes.  Where the other CTAs of the tile have left their parts already (it was their first tile), this one adds them to what it
+    // has and writes C; otherwise it leaves its own, and the last arriver adds up all of them.  All that needs a division is worked out in
+    // front, while the last MMAs run, and the parts of three CTAs come in one latency of the L2 (24 x 8192 x 22016, 2:4, 86 tiles on 148 CTAs:
+    // 21.2 us with the general code of finish_stripe at the end, 19.9 so; in pieces of 16 rows 20.3).
+    const uint32_t slot0 = 2u * (uint32_t)first_w + ((!p.split && shared_tile && vcol != stripe_begin32((uint32_t)first_w, U, P) / KB) ? 1u : 0u);
+    auto part_slot = [&](int q) { return slot_ptr(q == 0 ? slot0 : 2u * (uint32_t)(first_w + q)); };  // (see stripe_slot)
     if (w16 == 0 && lane == 0) *others_flag = shared_tile && ld_acquire_gpu(stripe_counter) == last_w - first_w ? 1 : 0;
     named_bar_sync(1, kAuxWarp0 * 32);  // (also: the drain is done with the tile before, which went through all output buffers)
     const bool onto = *others_flag != 0;
-    for (int c = g; c < pieces; c += 4) {
-      const int t = c % NT, b = c / NT * 2;
-      if (onto) {
-        gather(two, t, b, last_w - first_w + 1, (int)worker - first_w, [&](int q) { return stripe_slot(first_w + q, vcol); }, nullptr);
-      } else {
-        own_sums(two, t, b, f);
-        if (shared_tile)
-          to_slot(two, t, b, f, stripe_slot((int)worker, vcol));
-        else
-          to_c(two, t, b, f);
+    if (shared_tile && !onto) {
+      float4* mine = part_slot((int)worker - first_w);
+      for (int c = g; c < pieces; c += 4) {
+        own_sums(two, c % NT, c / NT * 2, f);
+        to_slot(two, c % NT, c / NT * 2, f, mine);
       }
+      named_bar_sync(1, kAuxWarp0 * 32);
+      if (w16 == 0 && lane == 0) *last_flag = atom_add_acq_rel_gpu(stripe_counter, 1) == last_w - first_w ? 1 : 0;
+      named_bar_sync(1, kAuxWarp0 * 32);
+      if (*last_flag == 0) return;
     }
-    if (onto) {
+    if (shared_tile) {
+      const int parts = last_w - first_w + 1, own = onto ? (int)worker - first_w : parts;
+      for (int c = g; c < units; c += 4) gather(c % NT, c / NT, parts, own, part_slot, nullptr);
       if (w16 == 0 && lane == 0) *stripe_counter = 0;
     } else {
-      finish_stripe(w16);
+      for (int c = g; c < pieces; c += 4) {
+        own_sums(two, c % NT, c / NT * 2, f);
+        to_c(two, c % NT, c / NT * 2, f);
+      }
     }
   };
 
