@@ -75,6 +75,7 @@ constexpr uint64_t kWaitLimitNs = MARLIN_WAIT_LIMIT_NS;
 // leaves out the copies of its second pipeline stage, so that the waits on that stage run into their limit and
 // the time-out path can be exercised without any fault.  The product library is built without the hooks.
 constexpr int kTestWithholdMagic = 0x57495448;
+constexpr int kTestLeaveMagic = 0x4c454156;  // stripes: a CTA leaves its part even where those of the others are there
 // BACKOFF_NS > 0: sleep between polls.  The copy-issuing warps use it: their waits are long and not urgent,
 // and a warp that polls flat out takes issue slots from the compute warps of its scheduler.
 template <int BACKOFF_NS = 0>

@@ -657,7 +657,11 @@ gemm_tc_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmap_a) {
     auto part_slot = [&](int q) { return slot_ptr(q == 0 ? slot0 : 2u * (uint32_t)(first_w + q)); };  // (see stripe_slot)
     if (w16 == 0 && lane == 0) *others_flag = shared_tile && ld_acquire_gpu(stripe_counter) == last_w - first_w ? 1 : 0;
     named_bar_sync(1, kAuxWarp0 * 32);  // (also: the drain is done with the tile before, which went through all output buffers)
+#ifdef MARLIN_TEST_HOOKS
+    const bool onto = *others_flag != 0 && p.status[7] != kTestLeaveMagic;
+#else
     const bool onto = *others_flag != 0;
+#endif
     if (shared_tile && !onto) {
       float4* mine = part_slot((int)worker - first_w);
       for (int c = g; c < pieces; c += 4) {

@@ -86,3 +86,25 @@ def test_an_expired_wait_is_reported_and_the_next_call_is_correct(marlin, test_l
     C2 = to_host(marlin.gemm(A, w, s, K, N, G, ws2))
     assert marlin.read_status(ws2) == 0
     assert oracle_lib.check_tolerance(C2, ref)[0] == 0
+
+
+# stripes: a CTA adds its part from tensor memory onto those of the others where they have come first, else leaves it in its slot for the last
+# arriver; the test build takes the second way always.  One scale per column, whose products are not exact: the bits must not tell.
+@pytest.mark.parametrize("M,K,N", [(24, 4096, 3072), (100, 2048, 6144), (300, 2048, 2048)])
+def test_parts_from_registers_and_from_slots_give_the_same_bits(marlin, test_lib, monkeypatch, M, K, N):
+    import torch
+    monkeypatch.setenv("MARLIN_B200_TC_SPLIT", "0")
+    case = inputs.make_dense(M, K, N, -1, seed=5 + M)
+    w, s = marlin.pack(to_dev(case.q_kpacked), to_dev(case.S), -1)
+    A = to_dev(case.A)
+    ws = marlin.new_workspace(M, K, N)
+    want = marlin.gemm(A, w, s, K, N, K, ws)
+    stream = torch.cuda.current_stream().cuda_stream
+    for leave in (0, 0x4c454156):
+        ws.zero_()
+        ws.view(torch.int32)[7] = leave
+        for _ in range(5):
+            C = torch.full((M, N), float("nan"), dtype=torch.float16, device="cuda")
+            assert test_lib.marlin_gemm(A.data_ptr(), w.data_ptr(), s.data_ptr(), C.data_ptr(), M, K, N, K, ws.data_ptr(), ws.numel(), stream) == 0
+            assert test_lib.marlin_read_status(ws.data_ptr(), stream) == 0
+            assert torch.equal(C, want)
