@@ -133,7 +133,7 @@ MARLIN_API int marlin_unpack_zeros(const void* z_packed, uint8_t* zeros, int K, 
  * weight, as in the paper's kernel).
  * Up to 16 rows the warp-level kernel runs, from 17 rows (from nine on layers of more than 2^26 weights with one scale
  * per column) a tcgen05 kernel.  That one takes all rows in one launch: above
- * 128 rows the layer is replicated in the numbering of the work units, once per slab of 128 rows (Section 3.4,
+ * 128 rows the layer is replicated in the numbering of the work units, once per slab of up to 128 rows (Section 3.4,
  * last paragraph), and the stripes of the CTAs run over (column tile, slab, k-block), so the weights come from
  * DRAM once and from the L2 after that.  Groups of 64 or 32 rows run on it at every batch size.
  * Partial sums are added in a fixed order everywhere: the same inputs give the same bits on every call.
@@ -237,7 +237,7 @@ MARLIN_API int marlin_unpack_sparse24(const void* w_packed, const void* meta_pac
 
 /* C = A . dequant(expand(W)) with the pruned positions contributing zero.  Layers whose N is a multiple of 256
  * run on the sparse tcgen05 instruction (tcgen05.mma.sp) at every batch size, all rows in one launch (slabs of
- * 128 rows as in marlin_gemm), reading the compressed weights from DRAM once; other N on the warp-level sparse
+ * rows as in marlin_gemm), reading the compressed weights from DRAM once; other N on the warp-level sparse
  * MMA in slabs of 16 rows. */
 MARLIN_API int marlin_gemm_sparse24(const void* A, const void* w_packed, const void* meta_packed,
                          const void* s_packed, void* C, int M, int K, int N, int group_size,

@@ -36,9 +36,9 @@
 // What bounds it: up to 64 rows the weights (8192 x 8192, 4-bit: 34 MB, 5.0 us at 6.8 TB/s), behind them the conversion (about
 // 240 cycles per 128 x 128 k-block and scheduler) and one hand-over between the warps per k-block (about 100 cycles each); at 128 rows
 // also the MMAs (64 cycles per 128 x 128 x 16); prefill from some hundreds of rows: the conversion again, and the power limit.
-// Measured on B200, cold weights, launches one behind the other: 8192 x 8192 at 32 / 64 / 128 rows 13.1 / 14.8 / 18.1 us (the kernel
-// with one role for conversion and drain before it: 15.2 / 17.0 / 21.5), at 1024 rows 107; 2:4 at 16 / 64 / 128 rows
-// 10.0 / 12.2 / 14.8 (11.6 / 14.0 / 17.2); 8-bit at 1 / 128 rows 14.5 / 20.1 (15.3 / 22.8).
+// Measured on B200, cold weights, launches one behind the other: 8192 x 8192 at 32 / 64 / 128 rows 12.8 / 14.6 / 17.7 us (the kernel
+// with one role for conversion and drain before it: 15.2 / 17.0 / 21.5); 2:4 at 16 / 64 / 128 rows 9.8 / 11.7 / 13.8
+// (11.6 / 14.0 / 17.2); 8-bit at one row 14.2 (15.3), at 100 rows 19.0.
 //
 // Partition: every column tile is cut into S k-ranges, one per CTA, where that keeps most SMs busy (one
 // epilogue per CTA, all CTAs alike); else even stripes over all units.  Fix-up of a shared tile: the CTAs of a

@@ -47,8 +47,11 @@ struct TcPlan {
 // The constants are a fit to launch times on B200 (launches one behind the other, from 64 rows on for 60 ms and more, so
 // that the power limit has its say: a 256-column tile reads the activations half as often, 8-bit, 2300 x 8192 x 8192 310 us against 352) of
 // every candidate on 1220 (layer, rows) pairs: 4-bit with groups of 128, 64 and 32 rows and with one scale, 2:4, 8-bit and deferred
-// scales, K and N from 1024 to 28672, 1 to 4096 rows.  The candidate it picks is on average 0.6 % slower than the
-// fastest one and more than 5 % on 36 pairs.  The constants before it (from about a dozen shapes, nothing per tile, the 8-bit ones
+// scales, K and N from 1024 to 28672, 1 to 4096 rows.  The candidate it picked was on average 0.6 % slower than the
+// fastest one and more than 5 % on 36 pairs.  The end of a launch (read-out by 16 warps, exchange in units of eight rows, sums of stripes) and the
+// slabs have become faster since, the constants are those from before: of 95 pairs timed on the kernel as it is, the pick is 1.4 % slower on
+// average, more than 5 % on nine (zero points, 49 x 8192 x 22272: 51 us in whole tiles, 38 in stripes; 22 x 4096 x 22016 18.5 / 16.8; 2:4, 1 x 4096 x
+// 22016 13.1 / 12.2).  The constants before it (from about a dozen shapes, nothing per tile, the 8-bit ones
 // scaled from 4-bit, 1.8 us for a small grid) missed by 2.6 % and, by more than 5 %, on 212 of 1198: 28672 x 8192 at 48 rows
 // 46 us, 35 now (256 columns and four k-ranges instead of 128 and two); 8-bit at 256 rows 145 / 113; 2:4, 1024 x 14336 at 128 rows
 // 11.5 / 8.0; 4096 x 22016 at 64 rows 18.5 / 14.4.  Zero points, whose conversion is longer, have k-blocks of their own: with those
